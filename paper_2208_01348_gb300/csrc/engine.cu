@@ -398,9 +398,11 @@ void set_grid(eels_ctx* c, const eels_grid* g) {
     L.contig = contig ? 1 : 0;
     L.nmat = maxm;
     L.px = make_plan(Mx); L.py = make_plan(My); L.pz = make_plan(Mz);
+    L.qx = make_plan2(Mx); L.qy = make_plan2(My); L.qz = make_plan2(Mz);
+    L.s32 = make_slab_plan(L, sizeof(float2));
+    L.s64 = make_slab_plan(L, sizeof(double2));
     L.tw64x = c->tw64[0].as<double2>(); L.tw64y = c->tw64[1].as<double2>(); L.tw64z = c->tw64[2].as<double2>();
     L.tw32x = c->tw32[0].as<float2>(); L.tw32y = c->tw32[1].as<float2>(); L.tw32z = c->tw32[2].as<float2>();
-    if (matvec_smem_bytes(L, true) == 0) throw Fail{EELS_E_UNSUPPORTED, "grid: FFT tiles do not fit shared memory"};
     CK(cudaStreamSynchronize(c->stream));
     c->has_grid = true;
     c->tuned = false;
@@ -657,6 +659,9 @@ MatvecArgs<Rl> mv_args(eels_ctx* c, int S, const cx<Rl>* x, cx<Rl>* y, const cx<
     return a;
 }
 
+// Most partial sums of x^T (A x) per system that a matvec of either precision writes.
+int dot_parts(const LatticeDev& L) { return std::max(matvec_dot_parts(L, false), matvec_dot_parts(L, true)); }
+
 template <typename Rl> const cx<Rl>* dr_of(eels_ctx* c);
 template <> const float2* dr_of<float>(eels_ctx* c) { return c->Dr32.as<float2>(); }
 template <> const double2* dr_of<double>(eels_ctx* c) { return c->Dr64.as<double2>(); }
@@ -668,9 +673,9 @@ int inner_solve(eels_ctx* c, int S, const eels_opts* o, double eps) {
     cudaStream_t st = c->stream;
     KrylovArgs<Rl> k = krylov_args<Rl>(c, S, o, eps);
     const bool bicg = o->solver == EELS_BICGSTAB, qmr2 = o->solver == EELS_QMR2;
-    // the three-pass matvec also returns the per-slab partial sums of x^T (A x)
-    const bool fused = !bicg && matvec_passes(c->L, sizeof(Rl) == 8) == 3;
-    k.nblk_a = fused ? 3 * c->L.Nx : k.nblk;
+    // the matvec also returns the per-block partial sums of x^T (A x)
+    const bool fused = !bicg;
+    k.nblk_a = fused ? matvec_dot_parts(c->L, sizeof(Rl) == 8) : k.nblk;
     if (bicg) launch_bicg_init<Rl>(k, st);
     else if (qmr2) launch_qmr2_init<Rl>(k, st);
     else launch_qmr_init<Rl>(k, st);
@@ -930,7 +935,7 @@ void krylov_dev(eels_ctx* c, int solver, const void* b, void* x, int S, double e
     const int nblk = (n3 + RED_CHUNK - 1) / RED_CHUNK;
     const size_t kvec = (size_t)S * n3 * sizeof(cx<Rl>);
     for (auto& v : c->kv) v.ensure(kvec);
-    c->part_a.ensure((size_t)S * std::max(nblk, 3 * c->L.Nx) * 4 * sizeof(double));
+    c->part_a.ensure((size_t)S * std::max(nblk, dot_parts(c->L)) * 4 * sizeof(double));
     c->part_b.ensure((size_t)S * nblk * 4 * sizeof(double));
     c->qmr.ensure((size_t)S * sizeof(QmrState));
     c->bicg.ensure((size_t)S * sizeof(BicgState));
@@ -1054,7 +1059,7 @@ int solve_impl(eels_ctx* c, const eels_opts* o, int n_energy, const double* ener
         c->u32.ensure((size_t)S * n3 * sizeof(float2));
         c->U.ensure((size_t)S * 3 * L.My * L.Nx * L.Mz * sizeof(double2));
         for (auto& b : c->kv) b.ensure(kvec);
-        c->part_a.ensure((size_t)S * std::max(nblk, 3 * L.Nx) * 4 * sizeof(double));
+        c->part_a.ensure((size_t)S * std::max(nblk, dot_parts(L)) * 4 * sizeof(double));
         c->part_b.ensure((size_t)S * nblk * 4 * sizeof(double));
         c->qmr.ensure((size_t)S * sizeof(QmrState));
         c->bicg.ensure((size_t)S * sizeof(BicgState));

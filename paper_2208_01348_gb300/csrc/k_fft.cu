@@ -7,10 +7,13 @@
 // lattice (separation (i - M) for the upper indices, zero at R = 0 and at
 // indices no separation reaches).  The input u is non-zero only on the
 // first Nx x Ny x Nz corner and only that corner of the output is needed, so
-// the forward transform runs z (Nx*Ny lines), then y (Nx*Mz lines), then x
-// (My*Mz lines, fused with the D-hat product and the inverse x transform),
-// and the inverse retraces y then z:  five passes over one scratch array
-// U[s][c][y][x][z] (z fastest), every pass coalesced along z or x.
+// a matvec is three passes over one scratch array U[s][c][y][x][z] (z
+// fastest): a slab pass (gather, y and z transforms of one x-slab), the x pass
+// (My*Mz lines: x transform, D-hat product, inverse x transform) and a slab
+// pass back (inverse z and y transforms, combination with x, scatter).  This
+// file holds the slab passes of 64 x 64 and 128 x 128 points in FP32, the D-hat
+// build and the launch of a matvec; k_slab.cuh and k_xline.cuh the passes of
+// any length, k_xreg.cu the x pass of 64 and 128 points in FP32.
 //
 // D-hat is stored on the octant 0 <= k <= M/2 only (6 (M/2+1)^3 values):
 // the diagonal components are even in each k and xy, xz, yz are odd in the
@@ -31,84 +34,6 @@ template <> __device__ __forceinline__ const double2* tw_of<double>(const Lattic
 }
 template <> __device__ __forceinline__ const float2* tw_of<float>(const LatticeDev& L, int axis) {
     return axis == 0 ? L.tw32x : (axis == 1 ? L.tw32y : L.tw32z);
-}
-
-// ---------------------------------------------------------------------------
-// Pass 1 (five-pass path): scatter the dipole vector onto the lattice (times
-// coef) and transform along z.  Block: W y-adjacent lines at fixed (s, c, ix).
-// ---------------------------------------------------------------------------
-template <typename Rl, int W>
-__global__ void __launch_bounds__(FFT_THREADS) k_zfwd(LatticeDev L, MatvecArgs<Rl> a) {
-    using C = cx<Rl>;
-    const int b = blockIdx.z, s = b / 3, c = b % 3;
-    if (a.active && !a.active[s]) return;
-    const int ix = blockIdx.y, iy0 = blockIdx.x * W;
-    const int Mz = L.Mz, ls = Mz + 1;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* tw = reinterpret_cast<C*>(smem_raw);
-    C* A = tw + Mz;
-    C* B = A + W * ls;
-    const C* twg = tw_of<Rl>(L, 2);
-    for (int t = threadIdx.x; t < Mz; t += blockDim.x) tw[t] = twg[t];
-    const C* xs = a.x + ((size_t)s * 3 + c) * L.N;
-    const double2* cf = a.coef + (size_t)s * EELS_MAX_MAT;
-    for (int t = threadIdx.x; t < W * Mz; t += blockDim.x) {
-        const int iz = t % Mz, w = t / Mz, iy = iy0 + w;
-        C v = mk<C>(0.0, 0.0);
-        if (iz < L.Nz && iy < L.Ny) {
-            const int dip = L.cellmap[((size_t)ix * L.Ny + iy) * L.Nz + iz];
-            if (dip >= 0) v = xs[dip] * cvt<C>(cf[L.mat[dip]]);
-        }
-        A[w * ls + iz] = v;
-    }
-    __syncthreads();
-    const C* r = fft_lines<false, false, W>(A, B, ls, 1, L.pz, tw);
-    C* U = a.U + (((size_t)s * 3 + c) * L.My * L.Nx + ix) * (size_t)Mz;
-    const size_t row = (size_t)L.Nx * Mz;
-    for (int t = threadIdx.x; t < W * Mz; t += blockDim.x) {
-        const int kz = t % Mz, w = t / Mz, iy = iy0 + w;
-        if (iy < L.Ny) U[(size_t)iy * row + kz] = r[w * ls + kz];
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Pass 5 (five-pass path): inverse z transform and gather:
-//   y = diag x - coef conv / M.
-// ---------------------------------------------------------------------------
-template <typename Rl, int W>
-__global__ void __launch_bounds__(FFT_THREADS) k_zinv(LatticeDev L, MatvecArgs<Rl> a, Rl invM) {
-    using C = cx<Rl>;
-    const int b = blockIdx.z, s = b / 3, c = b % 3;
-    if (a.active && !a.active[s]) return;
-    const int ix = blockIdx.y, iy0 = blockIdx.x * W;
-    const int Mz = L.Mz, ls = Mz + 1;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* tw = reinterpret_cast<C*>(smem_raw);
-    C* A = tw + Mz;
-    C* B = A + W * ls;
-    const C* twg = tw_of<Rl>(L, 2);
-    for (int t = threadIdx.x; t < Mz; t += blockDim.x) tw[t] = twg[t];
-    const C* U = a.U + (((size_t)s * 3 + c) * L.My * L.Nx + ix) * (size_t)Mz;
-    const size_t row = (size_t)L.Nx * Mz;
-    for (int t = threadIdx.x; t < W * Mz; t += blockDim.x) {
-        const int kz = t % Mz, w = t / Mz, iy = iy0 + w;
-        A[w * ls + kz] = iy < L.Ny ? U[(size_t)iy * row + kz] : mk<C>(0.0, 0.0);
-    }
-    __syncthreads();
-    const C* r = fft_lines<true, false, W>(A, B, ls, 1, L.pz, tw);
-    const C* xs = a.x + ((size_t)s * 3 + c) * L.N;
-    C* ys = a.y + ((size_t)s * 3 + c) * L.N;
-    const double2* cf = a.coef + (size_t)s * EELS_MAX_MAT;
-    const double2* dg = a.diag + (size_t)s * EELS_MAX_MAT;
-    for (int t = threadIdx.x; t < W * L.Nz; t += blockDim.x) {
-        const int iz = t % L.Nz, w = t / L.Nz, iy = iy0 + w;
-        if (iy >= L.Ny) continue;
-        const int dip = L.cellmap[((size_t)ix * L.Ny + iy) * L.Nz + iz];
-        if (dip < 0) continue;
-        const int m = L.mat[dip];
-        const C conv = invM * r[w * ls + iz];
-        ys[dip] = cvt<C>(dg[m]) * xs[dip] - cvt<C>(cf[m]) * conv;
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -161,212 +86,6 @@ __global__ void __launch_bounds__(FFT_THREADS) k_axis(cx<Rl>* data, int n1, int 
             const int w = t % W, i = t / W, i3 = i30 + w;
             if (i3 < n3) d[(size_t)i * stride + i3] = r[i * es + w];
         }
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Pass 3: forward x transform of the three components, product with the
-// symmetric D-hat tensor, inverse x transform.  Block: W z-adjacent lines
-// at fixed (s, ky); the 3W lines are interleaved in shared memory.
-// ---------------------------------------------------------------------------
-template <typename Rl, int W>
-__global__ void __launch_bounds__(FFT_THREADS) k_xpass(LatticeDev L, MatvecArgs<Rl> a) {
-    using C = cx<Rl>;
-    const int s = blockIdx.z;
-    if (a.active && !a.active[s]) return;
-    const int ky = blockIdx.y, kz0 = blockIdx.x * W;
-    const int Mx = L.Mx, Mz = L.Mz, Nx = L.Nx;
-    constexpr int NL = 3 * W;
-    constexpr int es = NL + 1;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* tw = reinterpret_cast<C*>(smem_raw);
-    C* A = tw + Mx;
-    C* B = A + Mx * es;
-    const C* twg = tw_of<Rl>(L, 0);
-    for (int t = threadIdx.x; t < Mx; t += blockDim.x) tw[t] = twg[t];
-    __syncthreads();
-    const size_t plane = (size_t)L.Nx * Mz;
-    C* U0 = a.U + ((size_t)s * 3 * L.My + ky) * plane;
-    const size_t cstride = (size_t)L.My * plane;
-    const C zero = mk<C>(0.0, 0.0);
-    // forward x transforms of the 3W lines, read straight from U (rows ix >= Nx are zero)
-    C* X = (L.px.nst % 2 == 0) ? B : A;   // the buffer the last forward stage does not read
-    C* Y = (X == A) ? B : A;
-    auto ld = [&](int l, int ix) -> C {
-        const int c = l / W, kz = kz0 + l % W;
-        return (ix < Nx && kz < Mz) ? U0[c * cstride + (size_t)ix * Mz + kz] : zero;
-    };
-    auto stX = [&](int l, int kx, C v) { X[kx * es + l] = v; };
-    fft_lines_io<false, true, NL>(A, B, 1, es, L.px, tw, ld, stX);
-    // D-hat product, in place in X
-    const int hx = Mx / 2, hy = L.My / 2, hz = Mz / 2;
-    const int kyr = ky <= hy ? ky : L.My - ky;
-    const Rl sy = ky <= hy ? (Rl)1 : (Rl)-1;
-    const size_t cs = (size_t)L.Hy * L.Hx * L.Hz;
-    const C* Ds = a.Dr + (size_t)a.sys_slot[s] * 6 * cs;
-    for (int t = threadIdx.x; t < W * Mx; t += blockDim.x) {
-        const int w = t % W, kx = t / W, kz = kz0 + w;
-        if (kz >= Mz) continue;
-        const int kxr = kx <= hx ? kx : Mx - kx;
-        const int kzr = kz <= hz ? kz : Mz - kz;
-        const Rl sx = kx <= hx ? (Rl)1 : (Rl)-1;
-        const Rl sz = kz <= hz ? (Rl)1 : (Rl)-1;
-        const size_t idx = ((size_t)kyr * L.Hx + kxr) * L.Hz + kzr;
-        const C dxx = Ds[idx], dxy = (sx * sy) * Ds[cs + idx], dxz = (sx * sz) * Ds[2 * cs + idx];
-        const C dyy = Ds[3 * cs + idx], dyz = (sy * sz) * Ds[4 * cs + idx], dzz = Ds[5 * cs + idx];
-        C* e = X + kx * es + w;
-        const C Xv = e[0], Yv = e[W], Zv = e[2 * W];
-        e[0] = dxx * Xv + dxy * Yv + dxz * Zv;
-        e[W] = dxy * Xv + dyy * Yv + dyz * Zv;
-        e[2 * W] = dxz * Xv + dyz * Yv + dzz * Zv;
-    }
-    __syncthreads();
-    // inverse x transforms, the first Nx outputs written straight back to U
-    auto ldX = [&](int l, int kx) -> C { return X[kx * es + l]; };
-    auto st = [&](int l, int ix, C v) {
-        const int c = l / W, kz = kz0 + l % W;
-        if (ix < Nx && kz < Mz) U0[c * cstride + (size_t)ix * Mz + kz] = v;
-    };
-    fft_lines_io<true, true, NL>(Y, X, 1, es, L.px, tw, ldX, st);
-}
-
-// The x pass for the common lengths Mx = 64 (8 x 8) and Mx = 128 (8 x 8 x 2)
-// with the stage descriptors known at compile time: the same shared-memory
-// Stockham stages and D-hat product as k_xpass, but every index division,
-// mask and loop bound folds to constants, and the block has one thread per
-// radix-8 butterfly of a stage (3W lines x MX/8).
-__host__ __device__ constexpr int cilog2(int v) { return (v > 0 && (v & (v - 1)) == 0) ? (v == 1 ? 0 : 1 + cilog2(v / 2)) : -1; }
-__host__ __device__ constexpr FftStage cstage(int len, int r, int ns) {
-    return FftStage{r, ns, cilog2(ns), len / r, cilog2(len / r), len / (ns * r)};
-}
-
-// First forward stage (sub-transform length 1, no twiddles) whose inputs
-// j + r L/R lie in the zero padding for r >= R/2 when HALF (the lattice fills
-// exactly the first half of the line): those inputs are compile-time zeros.
-template <int R, int NL, int LEN, bool HALF, typename C, class In, class Out>
-__device__ __forceinline__ void xstage_first(In in, Out out) {
-    constexpr int nb = LEN / R;
-    for (int t = threadIdx.x; t < NL * nb; t += blockDim.x) {
-        const int line = t % NL, j = t / NL;
-        C v[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = (!HALF || r < R / 2) ? in(line, j + r * nb) : mk<C>(0.0, 0.0);
-        Dft<R, false, C>::run(v);
-#pragma unroll
-        for (int r = 0; r < R; ++r) out(line, j * R + r, v[r]);
-    }
-}
-
-// Last inverse stage (sub-transform length L/R, twiddle stride 1): with HALF
-// only the outputs j + r L/R with r < R/2 (the lattice half) are formed.
-template <int R, int NL, int LEN, bool HALF, typename C, class In, class Out>
-__device__ __forceinline__ void xstage_last_inv(const C* __restrict__ tw, In in, Out out) {
-    constexpr int nb = LEN / R;
-    for (int t = threadIdx.x; t < NL * nb; t += blockDim.x) {
-        const int line = t % NL, j = t / NL;
-        C v[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = in(line, j + r * nb);
-#pragma unroll
-        for (int r = 1; r < R; ++r) {
-            C w = tw[r * j];
-            w.y = -w.y;
-            v[r] = v[r] * w;
-        }
-        Dft<R, true, C>::run(v);
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-            if (!HALF || r < R / 2) out(line, j + r * nb, v[r]);
-    }
-}
-
-template <int MX> struct XPlan;
-template <> struct XPlan<64> { static constexpr int n = 2, r[3] = {8, 8, 1}; };
-template <> struct XPlan<128> { static constexpr int n = 3, r[3] = {8, 8, 2}; };
-
-template <typename Rl, int W, int MX, bool HALF>
-__global__ void __launch_bounds__(3 * W * (MX / 8), (W == 16 && MX == 64 && sizeof(Rl) == 4) ? 4 : 1)
-k_xpassc(LatticeDev L, MatvecArgs<Rl> a) {
-    using C = cx<Rl>;
-    using P = XPlan<MX>;
-    constexpr int NT = 3 * W * (MX / 8);
-    constexpr FftStage S0 = cstage(MX, P::r[0], 1);
-    constexpr FftStage S1 = cstage(MX, P::r[1], P::r[0]);
-    constexpr FftStage S2 = cstage(MX, P::n == 3 ? P::r[2] : 2, P::r[0] * P::r[1]);
-    const int s = blockIdx.z;
-    if (a.active && !a.active[s]) return;
-    const int ky = blockIdx.y, kz0 = blockIdx.x * W;
-    const int Mz = L.Mz, Nx = L.Nx;
-    constexpr int NL = 3 * W;
-    constexpr int es = NL + 1;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* tw = reinterpret_cast<C*>(smem_raw);
-    C* A = tw + MX;
-    C* B = A + MX * es;
-    const C* twg = tw_of<Rl>(L, 0);
-    for (int t = threadIdx.x; t < MX; t += NT) tw[t] = twg[t];
-    __syncthreads();
-    const size_t plane = (size_t)Nx * Mz;
-    C* U0 = a.U + ((size_t)s * 3 * L.My + ky) * plane;
-    const size_t cstride = (size_t)L.My * plane;
-    const C zero = mk<C>(0.0, 0.0);
-    auto ld = [&](int l, int ix) -> C {
-        const int c = l / W, kz = kz0 + l % W;
-        return (ix < Nx && kz < Mz) ? U0[c * cstride + (size_t)ix * Mz + kz] : zero;
-    };
-    auto st = [&](int l, int ix, C v) {
-        const int c = l / W, kz = kz0 + l % W;
-        if (ix < Nx && kz < Mz) U0[c * cstride + (size_t)ix * Mz + kz] = v;
-    };
-    auto inA = [&](int l, int i) -> C { return A[i * es + l]; };
-    auto inB = [&](int l, int i) -> C { return B[i * es + l]; };
-    auto outA = [&](int l, int i, C v) { A[i * es + l] = v; };
-    auto outB = [&](int l, int i, C v) { B[i * es + l] = v; };
-    // forward x transforms of the 3W lines: U -> A -> B (-> A)
-    xstage_first<P::r[0], NL, MX, HALF, C>(ld, outA);
-    __syncthreads();
-    fft_stage_f<P::r[1], false, true, NL>(S1, tw, inA, outB);
-    __syncthreads();
-    if (P::n == 3) {
-        fft_stage_f<(P::n == 3 ? P::r[2] : 2), false, true, NL>(S2, tw, inB, outA);
-        __syncthreads();
-    }
-    C* X = P::n == 3 ? A : B;         // holds the spectrum
-    // D-hat product, in place
-    const int hy = L.My / 2, hz = Mz / 2;
-    const int kyr = ky <= hy ? ky : L.My - ky;
-    const Rl sy = ky <= hy ? (Rl)1 : (Rl)-1;
-    const size_t cs = (size_t)L.Hy * L.Hx * L.Hz;
-    const C* Ds = a.Dr + (size_t)a.sys_slot[s] * 6 * cs + (size_t)kyr * L.Hx * L.Hz;
-#pragma unroll 2
-    for (int t = threadIdx.x; t < W * MX; t += NT) {
-        const int w = t % W, kx = t / W, kz = kz0 + w;
-        if (kz >= Mz) continue;
-        const int kxr = kx <= MX / 2 ? kx : MX - kx;
-        const int kzr = kz <= hz ? kz : Mz - kz;
-        const Rl sx = kx <= MX / 2 ? (Rl)1 : (Rl)-1;
-        const Rl sz = kz <= hz ? (Rl)1 : (Rl)-1;
-        const C* d = Ds + (size_t)kxr * L.Hz + kzr;
-        const C dxx = d[0], dxy = (sx * sy) * d[cs], dxz = (sx * sz) * d[2 * cs];
-        const C dyy = d[3 * cs], dyz = (sy * sz) * d[4 * cs], dzz = d[5 * cs];
-        C* e = X + kx * es + w;
-        const C Xv = e[0], Yv = e[W], Zv = e[2 * W];
-        e[0] = dxx * Xv + dxy * Yv + dxz * Zv;
-        e[W] = dxy * Xv + dyy * Yv + dyz * Zv;
-        e[2 * W] = dxz * Xv + dyz * Yv + dzz * Zv;
-    }
-    __syncthreads();
-    // inverse x transforms back to U (first Nx outputs)
-    if (P::n == 3) {
-        fft_stage_f<P::r[0], true, true, NL>(S0, tw, inA, outB);
-        __syncthreads();
-        fft_stage_f<P::r[1], true, true, NL>(S1, tw, inB, outA);
-        __syncthreads();
-        xstage_last_inv<(P::n == 3 ? P::r[2] : 2), NL, MX, HALF, C>(tw, inA, st);
-    } else {
-        fft_stage_f<P::r[0], true, true, NL>(S0, tw, inB, outA);
-        __syncthreads();
-        xstage_last_inv<P::r[1], NL, MX, HALF, C>(tw, inA, st);
     }
 }
 
@@ -452,162 +171,6 @@ __global__ void k_extract(LatticeDev L, int n_slot, const double2* G, double2* D
 }
 
 // ---------------------------------------------------------------------------
-// Fused slab passes (used when a slab fits shared memory): one block owns
-// the x-slab ix of one (system, component).  Forward: gather the Ny x Nz
-// corner, transform the Nz columns along y (CW at a time, into the slab
-// buffer S[My][Nz]), then the My rows along z (CW at a time) and write the
-// rows of U contiguously.  Inverse: the reverse order, then combine with x
-// and scatter.  Dipoles are numbered slab-major (ix, iy, iz with iz
-// fastest), so each slab's dipoles are contiguous and every global access
-// is coalesced.  This turns the five passes into three.
-// ---------------------------------------------------------------------------
-// Row stride of the z-transform tile: runs of 8 elements of consecutive rows
-// fall in disjoint bank groups when the stride is 8 mod 16.
-__host__ __device__ __forceinline__ int slab_row_stride(int Mz) {
-    int p = (Mz - 1) + ((Mz - 1) >> 3) + 1;   // padded row length (one slot per 8 elements)
-    while (p % 16 != 8) ++p;
-    return p;
-}
-// Slab buffer S[My][Nz]: rows padded to a multiple of 16 elements, and bit 3
-// of the column index flipped on odd rows, so that the 8-element runs that
-// consecutive rows read or write fall in disjoint banks without widening the
-// rows.
-__host__ __device__ __forceinline__ int slab_s_stride(int Nz) { return (Nz + 15) / 16 * 16; }
-__device__ __forceinline__ int sidx(int y, int z, int sls) { return y * sls + (z ^ ((y & 1) << 3)); }
-
-template <typename Rl, int CW>
-__device__ __forceinline__ void slab_smem(unsigned char* raw, const LatticeDev& L, cx<Rl>*& twy, cx<Rl>*& twz,
-                                          cx<Rl>*& S, cx<Rl>*& A, cx<Rl>*& B) {
-    using C = cx<Rl>;
-    const int scr = max(L.My * (CW + 1), CW * slab_row_stride(L.Mz));
-    twy = reinterpret_cast<C*>(raw);
-    twz = twy + L.My;
-    S = twz + L.Mz;
-    A = S + L.My * slab_s_stride(L.Nz);
-    B = A + scr;
-    const C* gy = tw_of<Rl>(L, 1);
-    const C* gz = tw_of<Rl>(L, 2);
-    for (int t = threadIdx.x; t < L.My; t += blockDim.x) twy[t] = gy[t];
-    for (int t = threadIdx.x; t < L.Mz; t += blockDim.x) twz[t] = gz[t];
-}
-
-template <typename Rl, int CW>
-__global__ void __launch_bounds__(FFT_THREADS) k_slab_fwd(LatticeDev L, MatvecArgs<Rl> a) {
-    using C = cx<Rl>;
-    const int ix = blockIdx.x, b = blockIdx.y, s = b / 3, c = b % 3;
-    if (a.active && !a.active[s]) return;
-    const int My = L.My, Ny = L.Ny, Nz = L.Nz;
-    const int sls = slab_s_stride(Nz), es = CW + 1, rls = slab_row_stride(L.Mz);
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *twy, *twz, *S, *A, *B;
-    slab_smem<Rl, CW>(smem_raw, L, twy, twz, S, A, B);
-    __syncthreads();
-    const C* xs = a.x + ((size_t)s * 3 + c) * L.N;
-    const double2* cf = a.coef + (size_t)s * EELS_MAX_MAT;
-    const int* cm = L.cellmap + (size_t)ix * Ny * Nz;
-    const C zero = mk<C>(0.0, 0.0);
-    // y transforms of the Nz columns (CW at a time): gathered from x, into S
-    for (int iz0 = 0; iz0 < Nz; iz0 += CW) {
-        auto ld = [&](int l, int y) -> C {
-            const int iz = iz0 + l;
-            if (y >= Ny || iz >= Nz) return zero;
-            const int dip = cm[y * Nz + iz];
-            return dip >= 0 ? xs[dip] * cvt<C>(cf[L.mat[dip]]) : zero;
-        };
-        auto st = [&](int l, int y, C v) {
-            const int iz = iz0 + l;
-            if (iz < Nz) S[sidx(y, iz, sls)] = v;
-        };
-        fft_lines_io<false, true, CW>(A, B, 1, es, L.py, twy, ld, st);
-    }
-    // z transforms of the My rows (CW at a time): from S, rows written to U
-    C* U = a.U + (((size_t)s * 3 + c) * My * L.Nx + ix) * L.Mz;
-    const size_t row = (size_t)L.Nx * L.Mz;
-    for (int ky0 = 0; ky0 < My; ky0 += CW) {
-        auto ld = [&](int l, int z) -> C {
-            const int ky = ky0 + l;
-            return (z < Nz && ky < My) ? S[sidx(ky, z, sls)] : zero;
-        };
-        auto st = [&](int l, int z, C v) {
-            const int ky = ky0 + l;
-            if (ky < My) U[(size_t)ky * row + z] = v;
-        };
-        fft_lines_io<false, false, CW, true>(A, B, rls, 1, L.pz, twz, ld, st);
-    }
-}
-
-template <typename Rl, int CW>
-__global__ void __launch_bounds__(FFT_THREADS) k_slab_inv(LatticeDev L, MatvecArgs<Rl> a, Rl invM) {
-    using C = cx<Rl>;
-    const int ix = blockIdx.x, b = blockIdx.y, s = b / 3, c = b % 3;
-    if (a.active && !a.active[s]) return;
-    const int My = L.My, Ny = L.Ny, Nz = L.Nz;
-    const int sls = slab_s_stride(Nz), es = CW + 1, rls = slab_row_stride(L.Mz);
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *twy, *twz, *S, *A, *B;
-    slab_smem<Rl, CW>(smem_raw, L, twy, twz, S, A, B);
-    __syncthreads();
-    const C zero = mk<C>(0.0, 0.0);
-    // inverse z transforms of the My rows of U (CW at a time), first Nz outputs into S
-    const C* U = a.U + (((size_t)s * 3 + c) * My * L.Nx + ix) * L.Mz;
-    const size_t row = (size_t)L.Nx * L.Mz;
-    for (int ky0 = 0; ky0 < My; ky0 += CW) {
-        auto ld = [&](int l, int z) -> C {
-            const int ky = ky0 + l;
-            return ky < My ? U[(size_t)ky * row + z] : zero;
-        };
-        auto st = [&](int l, int z, C v) {
-            const int ky = ky0 + l;
-            if (ky < My && z < Nz) S[sidx(ky, z, sls)] = v;
-        };
-        fft_lines_io<true, false, CW, true>(A, B, rls, 1, L.pz, twz, ld, st);
-    }
-    // inverse y transforms of the Nz columns, first Ny outputs combined with x and scattered
-    const C* xs = a.x + ((size_t)s * 3 + c) * L.N;
-    C* ys = a.y + ((size_t)s * 3 + c) * L.N;
-    const double2* cf = a.coef + (size_t)s * EELS_MAX_MAT;
-    const double2* dg = a.diag + (size_t)s * EELS_MAX_MAT;
-    const int* cm = L.cellmap + (size_t)ix * Ny * Nz;
-    Rl dot[2] = {0, 0};
-    for (int iz0 = 0; iz0 < Nz; iz0 += CW) {
-        auto ld = [&](int l, int y) -> C {
-            const int iz = iz0 + l;
-            return iz < Nz ? S[sidx(y, iz, sls)] : zero;
-        };
-        auto st = [&](int l, int y, C v) {
-            const int iz = iz0 + l;
-            if (y >= Ny || iz >= Nz) return;
-            const int dip = cm[y * Nz + iz];
-            if (dip < 0) return;
-            const int m = L.mat[dip];
-            const C xv = xs[dip];
-            const C yv = cvt<C>(dg[m]) * xv - cvt<C>(cf[m]) * (invM * v);
-            ys[dip] = yv;
-            dot[0] += xv.x * yv.x - xv.y * yv.y;
-            dot[1] += xv.x * yv.y + xv.y * yv.x;
-        };
-        fft_lines_io<true, true, CW>(A, B, 1, es, L.py, twy, ld, st);
-    }
-    if (a.dot_part) {
-        // block sum in a fixed order (warp shuffles, then thread 0 over the warps)
-        for (int o = 16; o > 0; o >>= 1) {
-            dot[0] += __shfl_xor_sync(0xffffffffu, dot[0], o);
-            dot[1] += __shfl_xor_sync(0xffffffffu, dot[1], o);
-        }
-        Rl* red = reinterpret_cast<Rl*>(A);
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-        if (lane == 0) { red[2 * wid] = dot[0]; red[2 * wid + 1] = dot[1]; }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double s0 = 0, s1 = 0;
-            for (int i = 0; i < (int)(blockDim.x >> 5); ++i) { s0 += red[2 * i]; s1 += red[2 * i + 1]; }
-            double* p = a.dot_part + (((size_t)s * 3 + c) * L.Nx + ix) * 4;
-            p[0] = s0; p[1] = s1; p[2] = 0.0; p[3] = 0.0;
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------
 // Fused slab passes for My = Mz = L = 64 or 128 in FP32, register resident.
 //
 // A warp transforms 4 lines at once (fft_warp.cuh): lane = q + 4p holds, for
@@ -623,10 +186,6 @@ __global__ void __launch_bounds__(FFT_THREADS) k_slab_inv(LatticeDev L, MatvecAr
 // every column's occupied cells are contiguous in z, so a dipole's index is
 // the column's base plus iz (no cell-map load).
 // ---------------------------------------------------------------------------
-// Dipole at depth iz of a column whose occupied cells are contiguous:
-// ci = (index of the column's first dipole - its first iz, first iz, last iz + 1).
-__device__ __forceinline__ int col_dip(int4 ci, int iz) { return (iz >= ci.y && iz < ci.z) ? ci.x + iz : -1; }
-
 template <int R> struct SlabR {
     static constexpr int L = 8 * R;
     static constexpr int SLS = R == 8 ? 36 : 68;           // slab row stride
@@ -857,8 +416,6 @@ __global__ void __launch_bounds__(FFT_THREADS, R == 8 ? 4 : 2) k_slab_inv_r(Latt
 // ---------------------------------------------------------------------------
 static const size_t kSmemCap = 220 * 1024;
 
-template <typename Rl> static size_t smem_zpass(const LatticeDev& L, int W) { return (size_t)(L.Mz + 2 * W * (L.Mz + 1)) * sizeof(cx<Rl>); }
-template <typename Rl> static size_t smem_xpass(const LatticeDev& L, int W) { return (size_t)(L.Mx + 2 * L.Mx * (3 * W + 1)) * sizeof(cx<Rl>); }
 template <typename Rl> static size_t smem_axis(int Lf, int W, int axis) {
     return axis == 3 ? (size_t)(Lf + 2 * W * (Lf + 1)) * sizeof(cx<Rl>) : (size_t)(Lf + 2 * Lf * (W + 1)) * sizeof(cx<Rl>);
 }
@@ -898,65 +455,6 @@ static void axis_launch(cx<Rl>* data, int nb, int n1, int n2, int n3, int in_len
     if (W == 32) axis_launch_w<Rl, 32, INV, AXIS>(data, nb, n1, n2, n3, in_len, out_len, p, tw, active, per_sys, st);
     else if (W == 16) axis_launch_w<Rl, 16, INV, AXIS>(data, nb, n1, n2, n3, in_len, out_len, p, tw, active, per_sys, st);
     else axis_launch_w<Rl, 8, INV, AXIS>(data, nb, n1, n2, n3, in_len, out_len, p, tw, active, per_sys, st);
-}
-
-template <typename Rl> static const cx<Rl>* host_tw(const LatticeDev& L, int axis);
-template <> const double2* host_tw<double>(const LatticeDev& L, int axis) { return axis == 0 ? L.tw64x : (axis == 1 ? L.tw64y : L.tw64z); }
-template <> const float2* host_tw<float>(const LatticeDev& L, int axis) { return axis == 0 ? L.tw32x : (axis == 1 ? L.tw32y : L.tw32z); }
-
-template <typename Rl, int W>
-static void zpass_launch(const LatticeDev& L, const MatvecArgs<Rl>& a, bool inv, cudaStream_t st) {
-    dim3 grid((L.Ny + W - 1) / W, L.Nx, a.S * 3);
-    const size_t sm = smem_zpass<Rl>(L, W);
-    count_launch();
-    if (!inv) k_zfwd<Rl, W><<<grid, FFT_THREADS, sm, st>>>(L, a);
-    else k_zinv<Rl, W><<<grid, FFT_THREADS, sm, st>>>(L, a, (Rl)(1.0 / ((double)L.Mx * L.My * L.Mz)));
-}
-
-template <typename Rl, int W>
-static void xpass_launch(const LatticeDev& L, const MatvecArgs<Rl>& a, cudaStream_t st) {
-    dim3 grid((L.Mz + W - 1) / W, L.My, a.S);
-    count_launch();
-    const auto& px = L.px;
-    const bool x64 = L.Mx == 64 && px.nst == 2 && px.st[0].R == 8 && px.st[1].R == 8;
-    const bool x128 = L.Mx == 128 && px.nst == 3 && px.st[0].R == 8 && px.st[1].R == 8 && px.st[2].R == 2;
-    const bool half = 2 * L.Nx == L.Mx;             // the lattice fills exactly half of each line
-    if (x64) {
-        if (half) k_xpassc<Rl, W, 64, true><<<grid, 3 * W * 8, smem_xpass<Rl>(L, W), st>>>(L, a);
-        else k_xpassc<Rl, W, 64, false><<<grid, 3 * W * 8, smem_xpass<Rl>(L, W), st>>>(L, a);
-        return;
-    }
-    if constexpr (W <= 16) {                         // 3W x 16 threads per block
-        if (x128) {
-            if (half) k_xpassc<Rl, W, 128, true><<<grid, 3 * W * 16, smem_xpass<Rl>(L, W), st>>>(L, a);
-            else k_xpassc<Rl, W, 128, false><<<grid, 3 * W * 16, smem_xpass<Rl>(L, W), st>>>(L, a);
-            return;
-        }
-    }
-    k_xpass<Rl, W><<<grid, FFT_THREADS, smem_xpass<Rl>(L, W), st>>>(L, a);
-}
-
-template <typename Rl, int CW> static size_t smem_slab(const LatticeDev& L) {
-    const size_t scr = (size_t)std::max(L.My * (CW + 1), CW * slab_row_stride(L.Mz));
-    return ((size_t)L.My + L.Mz + (size_t)L.My * slab_s_stride(L.Nz) + 2 * scr) * sizeof(cx<Rl>);
-}
-
-// Widest column tile whose fused-slab shared memory fits one block (0: none).
-template <typename Rl> static int pick_slab(const LatticeDev& L) {
-    if (smem_slab<Rl, 32>(L) <= 110 * 1024) return 32;
-    if (smem_slab<Rl, 16>(L) <= 110 * 1024) return 16;
-    if (smem_slab<Rl, 16>(L) <= kSmemCap) return 16;
-    if (smem_slab<Rl, 8>(L) <= kSmemCap) return 8;
-    return 0;
-}
-
-template <typename Rl, int CW>
-static void slab_launch(const LatticeDev& L, const MatvecArgs<Rl>& a, bool inv, cudaStream_t st) {
-    dim3 grid(L.Nx, a.S * 3);
-    const size_t sm = smem_slab<Rl, CW>(L);
-    count_launch();
-    if (!inv) k_slab_fwd<Rl, CW><<<grid, FFT_THREADS, sm, st>>>(L, a);
-    else k_slab_inv<Rl, CW><<<grid, FFT_THREADS, sm, st>>>(L, a, (Rl)(1.0 / ((double)L.Mx * L.My * L.Mz)));
 }
 
 // Register-resident slab kernels: FP32 with 64- or 128-point y and z transforms.
@@ -1008,29 +506,21 @@ template <> bool slab_reg_launch<float>(const LatticeDev& L, const MatvecArgs<fl
     return false;
 }
 
-template <typename Rl> static void slab_launch_any(const LatticeDev& L, const MatvecArgs<Rl>& a, bool inv, int cw,
+template <typename Rl> static void slab_launch_any(const LatticeDev& L, const MatvecArgs<Rl>& a, bool inv,
                                                    cudaStream_t st) {
     if (slab_reg_launch<Rl>(L, a, inv, st)) return;
-    if (cw == 32) slab_launch<Rl, 32>(L, a, inv, st);
-    else if (cw == 16) slab_launch<Rl, 16>(L, a, inv, st);
-    else slab_launch<Rl, 8>(L, a, inv, st);
+    launch_slab<Rl>(L, a, inv, st);
 }
 
-// Widest x-pass tile (W lines per component) whose two buffers fit a
-// quarter of an SM's shared memory, so that four blocks are resident.
+// Widest x-pass tile (W lines per component) whose buffer fits a quarter of
+// an SM's shared memory, so that four blocks are resident.
 template <typename Rl> static int pick_xpass_w(const LatticeDev& L) {
     for (int W : {32, 16, 8})
-        if (smem_xpass<Rl>(L, W) <= 56 * 1024) return W;
-    return pick_w([&](int w) { return smem_xpass<Rl>(L, w); });
+        if (6 * (size_t)W * L.Mx * sizeof(cx<Rl>) <= 56 * 1024) return W;
+    return 8;
 }
 
 template <typename Rl> static int tuned_w(const LatticeDev& L) { return sizeof(Rl) == 4 ? L.xw32 : L.xw64; }
-
-template <typename Rl> static void xpass_w(const LatticeDev& L, const MatvecArgs<Rl>& a, int wx, cudaStream_t st) {
-    if (wx == 32) xpass_launch<Rl, 32>(L, a, st);
-    else if (wx == 16) xpass_launch<Rl, 16>(L, a, st);
-    else xpass_launch<Rl, 8>(L, a, st);
-}
 
 template <typename Rl>
 int autotune_xpass(const LatticeDev& L, const MatvecArgs<Rl>& a, cudaStream_t st) {
@@ -1041,10 +531,10 @@ int autotune_xpass(const LatticeDev& L, const MatvecArgs<Rl>& a, cudaStream_t st
     if (cudaEventCreate(&e1) != cudaSuccess) { cudaEventDestroy(e0); return best; }
     bool first = true;
     for (int w : {8, 16, 32}) {
-        if (smem_xpass<Rl>(L, w) > kSmemCap) continue;
-        xpass_w<Rl>(L, a, w, st);                   // warm-up
+        if (!xline_fits<Rl>(L, w)) continue;
+        launch_xline<Rl>(L, a, w, st);              // warm-up
         cudaEventRecord(e0, st);
-        for (int r = 0; r < 3; ++r) xpass_w<Rl>(L, a, w, st);
+        for (int r = 0; r < 3; ++r) launch_xline<Rl>(L, a, w, st);
         cudaEventRecord(e1, st);
         float ms = 0.f;
         if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) break;
@@ -1061,50 +551,21 @@ template <typename Rl> static void xpass_any(const LatticeDev& L, const MatvecAr
     if constexpr (sizeof(Rl) == 4) {
         if (launch_xpass_reg(L, a, st)) return;
     }
-    const int wx = tuned_w<Rl>(L) ? tuned_w<Rl>(L) : pick_xpass_w<Rl>(L);
-    if (wx == 32) xpass_launch<Rl, 32>(L, a, st);
-    else if (wx == 16) xpass_launch<Rl, 16>(L, a, st);
-    else xpass_launch<Rl, 8>(L, a, st);
+    launch_xline<Rl>(L, a, tuned_w<Rl>(L) ? tuned_w<Rl>(L) : pick_xpass_w<Rl>(L), st);
 }
 
 template <typename Rl>
-bool launch_matvec(const LatticeDev& L, const MatvecArgs<Rl>& a, cudaStream_t st) {
-    const int cw = pick_slab<Rl>(L);
-    if (cw) {   // three passes: slab (gather, y, z) -> x * D-hat * x -> slab (z, y, scatter)
-        slab_launch_any<Rl>(L, a, false, cw, st);
-        xpass_any<Rl>(L, a, st);
-        slab_launch_any<Rl>(L, a, true, cw, st);
-        return a.dot_part != nullptr;
-    }
-    const int wz = pick_w([&](int w) { return smem_zpass<Rl>(L, w); });
-    if (wz == 32) zpass_launch<Rl, 32>(L, a, false, st);
-    else if (wz == 16) zpass_launch<Rl, 16>(L, a, false, st);
-    else zpass_launch<Rl, 8>(L, a, false, st);
-    axis_launch<Rl, false, 1>(a.U, a.S * 3, L.My, L.Nx, L.Mz, L.Ny, L.My, L.py, host_tw<Rl>(L, 1), a.active, 3, st);
+void launch_matvec(const LatticeDev& L, const MatvecArgs<Rl>& a, cudaStream_t st) {
+    // slab (gather, y, z) -> x * D-hat * x -> slab (z, y, scatter)
+    slab_launch_any<Rl>(L, a, false, st);
     xpass_any<Rl>(L, a, st);
-    axis_launch<Rl, true, 1>(a.U, a.S * 3, L.My, L.Nx, L.Mz, L.My, L.Ny, L.py, host_tw<Rl>(L, 1), a.active, 3, st);
-    if (wz == 32) zpass_launch<Rl, 32>(L, a, true, st);
-    else if (wz == 16) zpass_launch<Rl, 16>(L, a, true, st);
-    else zpass_launch<Rl, 8>(L, a, true, st);
-    return false;
+    slab_launch_any<Rl>(L, a, true, st);
 }
 
 template <typename Rl, int W> static void prepare_w() {
-    allow_smem(k_zfwd<Rl, W>);
-    allow_smem(k_zinv<Rl, W>);
-    allow_smem(k_xpass<Rl, W>);
-    allow_smem(k_xpassc<Rl, W, 64, true>);
-    allow_smem(k_xpassc<Rl, W, 64, false>);
-    if constexpr (W <= 16) {
-        allow_smem(k_xpassc<Rl, W, 128, true>);
-        allow_smem(k_xpassc<Rl, W, 128, false>);
-    }
     allow_smem(k_axis<Rl, W, false, 1>);
-    allow_smem(k_axis<Rl, W, true, 1>);
     allow_smem(k_axis<Rl, W, false, 2>);
     allow_smem(k_axis<Rl, W, false, 3>);
-    allow_smem(k_slab_fwd<Rl, W>);
-    allow_smem(k_slab_inv<Rl, W>);
 }
 
 void prepare_far_kernels();
@@ -1130,25 +591,19 @@ void prepare_kernels() {
     allow_smem(k_slab_inv_r<16, false, true>);
     allow_smem(k_slab_inv_r<16, false, false>);
     prepare_far_kernels();
+    prepare_slab_kernels<float>();
+    prepare_slab_kernels<double>();
+    prepare_xline_kernels<float>();
+    prepare_xline_kernels<double>();
     prepare_xreg_kernels();
 }
 
-template bool launch_matvec<float>(const LatticeDev&, const MatvecArgs<float>&, cudaStream_t);
-template bool launch_matvec<double>(const LatticeDev&, const MatvecArgs<double>&, cudaStream_t);
+template void launch_matvec<float>(const LatticeDev&, const MatvecArgs<float>&, cudaStream_t);
+template void launch_matvec<double>(const LatticeDev&, const MatvecArgs<double>&, cudaStream_t);
 
-int matvec_passes(const LatticeDev& L, bool fp64) {
-    return (fp64 ? pick_slab<double>(L) : pick_slab<float>(L)) ? 3 : 5;
-}
-
-size_t matvec_smem_bytes(const LatticeDev& L, bool fp64) {
-    if (fp64) {
-        const int wx = pick_xpass_w<double>(L);
-        const int wz = pick_w([&](int w) { return smem_zpass<double>(L, w); });
-        if (!wx || !wz) return 0;
-        return smem_xpass<double>(L, wx);
-    }
-    const int wx = pick_xpass_w<float>(L);
-    return wx ? smem_xpass<float>(L, wx) : 0;
+static bool slab_reg(const LatticeDev& L) { return (L.My == 64 && L.Mz == 64) || (L.My == 128 && L.Mz == 128); }
+int matvec_dot_parts(const LatticeDev& L, bool fp64) {
+    return 3 * L.Nx * (fp64 ? L.s64.CL : slab_reg(L) ? 1 : L.s32.CL);
 }
 
 void launch_dhat_build(const LatticeDev& L, int n_slot, const double2* kappa, double2* G, double2* Dr64, float2* Dr32,

@@ -1,0 +1,129 @@
+// Shared-memory x pass (see xline.cuh), one kernel per padded length.
+//
+// Block: W z-adjacent lines of the three components at fixed ky, for up to
+// spb consecutive systems.  In FP32 the D-hat rows of those lines (octant
+// kx', six components) are copied into shared memory while step 1 runs, once
+// per D-hat slot (the beams of an energy share it); FP64 is bound by its
+// arithmetic and reads D-hat where it needs it, leaving the shared memory to
+// more blocks.  Two block barriers per system:
+// step 1 reads U, the middle step runs in registers (end of the forward
+// transform, D-hat product, start of the inverse transform), step 2 writes U;
+// step 2 reads the places that the same thread's next step 1 writes.
+//
+// FP32 is bound by latency (12 warps per SM at 160 points: shared memory), FP64
+// by its pipe.  160-point lines, 4 systems of 79^3 cells: 0.27 ms, against
+// 0.37 ms for one thread per butterfly of three run-time stages with D-hat
+// read from L2 in the product (0.31 ms with the middle in registers but D-hat
+// still read there).
+#pragma once
+#include <cuda_pipeline.h>
+
+#include <algorithm>
+
+#include "kernels.h"
+#include "xline.cuh"
+
+namespace eels {
+
+template <typename Rl> __device__ __forceinline__ const cx<Rl>* xline_tw(const LatticeDev& L);
+template <> __device__ __forceinline__ const double2* xline_tw<double>(const LatticeDev& L) { return L.tw64x; }
+template <> __device__ __forceinline__ const float2* xline_tw<float>(const LatticeDev& L) { return L.tw32x; }
+
+template <typename Rl, int RE, int RO>
+__global__ void __launch_bounds__(256, sizeof(Rl) == 4 && RO <= 10 ? (RO <= 6 ? 3 : 2) : 1)
+k_xline(LatticeDev L, MatvecArgs<Rl> a, int lgw) {
+    using C = cx<Rl>;
+    constexpr int LEN = RE * RO, HX = LEN / 2 + 1;
+    const int s0 = blockIdx.z * a.spb, s1 = min(a.S, s0 + a.spb);
+    const int W = 1 << lgw, ky = blockIdx.y, kz0 = blockIdx.x << lgw;
+    const int Mz = L.Mz, Nx = L.Nx;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C* tw = reinterpret_cast<C*>(smem_raw);             // w^(r j) at [r][j]
+    C* A = tw + LEN;                                    // [LEN][3][W]
+    C* D = A + 3 * LEN * W;                             // [6][HX][W] (FP32)
+    constexpr bool STAGE = sizeof(Rl) == 4;
+    const C* twg = xline_tw<Rl>(L);
+    for (int t = threadIdx.x; t < LEN; t += blockDim.x) tw[t] = twg[(t / RE) * (t % RE)];
+    const size_t plane = (size_t)Nx * Mz, cstride = (size_t)L.My * plane;
+    const int nw = min(W, Mz - kz0), hz = Mz / 2;
+    const bool ny = ky > L.My / 2;
+    const size_t cs = (size_t)L.Hy * L.Hx * L.Hz;
+    int cur = -1;
+    for (int s = s0; s < s1; ++s) {
+        if (a.active && !a.active[s]) continue;
+        const int slot = a.sys_slot[s];
+        const C* Ds = a.Dr + (size_t)slot * 6 * cs + (size_t)(ny ? L.My - ky : ky) * L.Hx * L.Hz;
+        if (STAGE && slot != cur) {                     // every thread is past the middle step that read D
+            for (int t = threadIdx.x; t < 6 * HX * W; t += blockDim.x) {
+                const int w = t & (W - 1), q = t >> lgw, c = q / HX, kx = q - c * HX, kz = kz0 + w;
+                if (w < nw)
+                    __pipeline_memcpy_async(D + t, Ds + c * cs + (size_t)kx * L.Hz + (kz > hz ? Mz - kz : kz), sizeof(C));
+            }
+            cur = slot;
+        }
+        C* U0 = a.U + ((size_t)s * 3 * L.My + ky) * plane + kz0;
+        xline_1<RE, RO>(A, lgw, Nx, threadIdx.x, blockDim.x, [&](int c, int w, int ix) -> C {
+            return w < nw ? U0[c * cstride + (size_t)ix * Mz + w] : mk<C>(0.0, 0.0);
+        });
+        if (STAGE) {
+            __pipeline_commit();
+            __pipeline_wait_prior(0);
+        }
+        __syncthreads();
+        xline_mid<RE, RO>(A, lgw, nw, tw, threadIdx.x, blockDim.x, [&](int w, int kx, C (&g)[6]) {
+            const int kz = kz0 + w, kxr = kx > LEN / 2 ? LEN - kx : kx;
+            const bool nx = kx > LEN / 2, nz = kz > hz;
+            const C* d = STAGE ? D + (kxr << lgw) + w : Ds + (size_t)kxr * L.Hz + (nz ? Mz - kz : kz);
+            const size_t st = STAGE ? (size_t)(HX << lgw) : cs;
+            g[0] = d[0];
+            g[1] = flip_c(d[st], nx != ny);
+            g[2] = flip_c(d[2 * st], nx != nz);
+            g[3] = d[3 * st];
+            g[4] = flip_c(d[4 * st], ny != nz);
+            g[5] = d[5 * st];
+        });
+        __syncthreads();
+        xline_2<RE, RO>(A, lgw, Nx, threadIdx.x, blockDim.x, [&](int c, int w, int ix, C v) {
+            if (w < nw) U0[c * cstride + (size_t)ix * Mz + w] = v;
+        });
+    }
+}
+
+template <typename Rl> static size_t xline_smem(const LatticeDev& L, int w) {
+    return (size_t)(L.Mx + 3 * w * L.Mx + (sizeof(Rl) == 4 ? 6 * w * (L.Mx / 2 + 1) : 0)) * sizeof(cx<Rl>);
+}
+template <typename Rl> bool xline_fits(const LatticeDev& L, int w) { return xline_smem<Rl>(L, w) <= 224 * 1024; }
+
+template <typename Rl> void launch_xline(const LatticeDev& L, const MatvecArgs<Rl>& a, int w, cudaStream_t st) {
+    int lgw = 0;
+    while ((2 << lgw) <= w) ++lgw;
+    // a grid that leaves SMs idle takes narrower tiles (the lines do not depend on the tile they are in):
+    // 144 blocks of 4 lines instead of 72 of 8 for one 12^3 system
+    while (lgw > 1 && (long long)((L.Mz + (1 << lgw) - 1) >> lgw) * L.My * a.S < 100) --lgw;
+    // systems per block: several when they can share D-hat and the grid stays large
+    const int tiles = ((L.Mz + (1 << lgw) - 1) >> lgw) * L.My;
+    MatvecArgs<Rl> b = a;
+    b.spb = std::max(1, std::min(a.spb, a.S));
+    while (b.spb > 1 && (long long)tiles * ((a.S + b.spb - 1) / b.spb) < 1216) b.spb /= 2;
+    const dim3 grid((L.Mz + (1 << lgw) - 1) >> lgw, L.My, (a.S + b.spb - 1) / b.spb);
+    const int nthr = std::min(256, std::max(64, ((L.qx.Re << lgw) + 31) / 32 * 32));
+    const size_t sm = xline_smem<Rl>(L, 1 << lgw);
+    count_launch();
+    switch (L.Mx) {
+#define XL(RE, RO) case RE * RO: k_xline<Rl, RE, RO><<<grid, nthr, sm, st>>>(L, b, lgw); break;
+        EELS_PLANS(XL)
+#undef XL
+        default: break;
+    }
+}
+
+template <typename Rl> void prepare_xline_kernels() {
+#define XL(RE, RO)                                                                                         \
+    cudaFuncSetAttribute(k_xline<Rl, RE, RO>, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);  \
+    cudaFuncSetAttribute(k_xline<Rl, RE, RO>, cudaFuncAttributePreferredSharedMemoryCarveout,            \
+                         (int)cudaSharedmemCarveoutMaxShared);
+    EELS_PLANS(XL)
+#undef XL
+}
+
+}  // namespace eels

@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "dft.cuh"
 #include "fft.cuh"
 
 namespace eels {
@@ -20,6 +21,17 @@ extern thread_local bool g_capturing;
 inline void count_launch(int n = 1) {
     if (!g_capturing) g_kernel_launches += n;
 }
+
+// Split of a slab pass (k_slab.cu) over the blocks of a cluster: chosen from
+// the lattice alone, so that a system's sums do not depend on the batch.
+struct SlabPlan {
+    int CL;                       // blocks per slab
+    int cpc, rpc;                 // columns iz and rows ky per block
+    int sls;                      // row stride of a block's columns S[My][sls]
+    int G;                        // rows a warp transforms at a time
+    int nthr;
+    FastDiv dcpc;                 // division by cpc
+};
 
 // Lattice description shared by every kernel (device pointers).
 struct LatticeDev {
@@ -36,11 +48,17 @@ struct LatticeDev {
     const double* igt;            // D-hat build only: cell tables of the igt_so interaction (igt.cu), or
                                   // nullptr for point dipoles
     FftPlan px, py, pz;
+    Plan2 qx, qy, qz;
+    SlabPlan s32, s64;            // slab passes in FP32 and FP64
     int xw32, xw64;               // x-pass tile width chosen by the autotuner (0: size heuristic)
     int xmode;                    // register x pass: 0 choose by availability, 1 direct loads, 2 tensor copies
     const double2* tw64x; const double2* tw64y; const double2* tw64z;   // exp(-2 pi i t / M)
     const float2* tw32x; const float2* tw32y; const float2* tw32z;
 };
+
+// Dipole at depth iz of a column whose occupied cells are contiguous:
+// ci = (index of the column's first dipole - its first iz, first iz, last iz + 1).
+__host__ __device__ __forceinline__ int col_dip(int4 ci, int iz) { return (iz >= ci.y && iz < ci.z) ? ci.x + iz : -1; }
 
 // y = diag[m] x - coef[m] * conv(coef[m'] x) / M for a batch of systems.
 // conv(u)_i = sum_{j != i} G~'(r_i - r_j) u_j evaluated by zero-padded FFT.
@@ -55,8 +73,8 @@ struct MatvecArgs {
     const double2* coef;          // [S][EELS_MAX_MAT]
     const double2* diag;          // [S][EELS_MAX_MAT]
     const int* active;            // [S] or nullptr
-    double* dot_part;             // optional [S][3 Nx][4]: per-slab sum x.y (unconjugated), written by the
-                                  // three-pass path's last kernel
+    double* dot_part;             // optional [S][matvec_dot_parts][4]: per-block sum x.y (unconjugated), written by
+                                  // the last kernel
     const float2* Dx;             // FP32 D-hat [slot][Hy][Hz][6][Hx] (register x pass), or nullptr
     int S;
     int spb;                      // systems per x-pass block (consecutive systems that usually share a
@@ -71,9 +89,18 @@ constexpr int IGT_NEAR = 3;
 constexpr double IGT_C1 = 2.3800773639795505;   // integral of 1/|u| over the unit cube: 3 ln(2 + sqrt 3) - pi/2
 const std::vector<double>& igt_tables();
 
-// Returns true when a.dot_part was filled (three-pass path).
+Plan2 make_plan2(int L);
+SlabPlan make_slab_plan(const LatticeDev& L, size_t el);   // el: bytes of a complex element
+size_t slab_smem(const LatticeDev& L, const SlabPlan& p, size_t el);
+template <typename Rl> void prepare_slab_kernels();
+// Slab pass of any y and z length (forward: gather to U; inverse: U to y).
 template <typename Rl>
-bool launch_matvec(const LatticeDev& L, const MatvecArgs<Rl>& a, cudaStream_t st);
+void launch_slab(const LatticeDev& L, const MatvecArgs<Rl>& a, bool inv, cudaStream_t st);
+// Partial sums of x^T (A x) per system that launch_matvec writes to dot_part.
+int matvec_dot_parts(const LatticeDev& L, bool fp64);
+
+template <typename Rl>
+void launch_matvec(const LatticeDev& L, const MatvecArgs<Rl>& a, cudaStream_t st);
 
 // D-hat build for n_slot energies: kappa[slot] = k d (complex).  G scratch
 // [n_slot][6][My][Mx][Mz] FP64; outputs reduced D-hat FP64 and FP32.
@@ -99,14 +126,17 @@ void autotune_xreg(const LatticeDev& L, const MatvecArgs<float>& a, int max_spb,
 // one left its kernel's results incomplete).  Reading it synchronises the device.
 unsigned int wait_timeouts();
 
-size_t matvec_smem_bytes(const LatticeDev& L, bool fp64);
+// Shared-memory x pass of any length, w kz-adjacent lines per block (a power
+// of two; narrower when the grid would leave SMs idle).
+template <typename Rl> bool xline_fits(const LatticeDev& L, int w);
+template <typename Rl> void launch_xline(const LatticeDev& L, const MatvecArgs<Rl>& a, int w, cudaStream_t st);
+template <typename Rl> void prepare_xline_kernels();
 // Times the x pass with every tile width whose shared memory fits, on the
 // systems of a (CUDA events on st; not during a stream capture), and returns
 // the fastest width.  The x pass transforms a.U in place: its contents are
 // lost.
 template <typename Rl>
 int autotune_xpass(const LatticeDev& L, const MatvecArgs<Rl>& a, cudaStream_t st);
-int matvec_passes(const LatticeDev& L, bool fp64);   // 3 (fused slabs) or 5
 
 // Raise the dynamic shared-memory limit of every kernel instance (call once
 // per device before any launch or stream capture).
