@@ -116,38 +116,6 @@ int pad_len_x(int n) {
     return good_fft_len(n);
 }
 
-FftPlan make_plan(int L) {
-    FftPlan p{};
-    p.L = L;
-    int r = L;
-    std::vector<int> rad;
-    // power-of-two radices first (largest first: fewer passes over shared
-    // memory, and Ns stays a power of two for shift/mask indexing), then 3, 5, 7
-    while (r % 8 == 0) { rad.push_back(8); r /= 8; }
-    while (r % 4 == 0) { rad.push_back(4); r /= 4; }
-    while (r % 2 == 0) { rad.push_back(2); r /= 2; }
-    for (int q : {3, 5, 7}) while (r % q == 0) { rad.push_back(q); r /= q; }
-    auto log2_or_neg = [](int v) {
-        if (v <= 0 || (v & (v - 1))) return -1;
-        int s = 0;
-        while ((1 << s) < v) ++s;
-        return s;
-    };
-    p.nst = (int)rad.size();
-    int Ns = 1;
-    for (int i = 0; i < p.nst; ++i) {
-        FftStage& sd = p.st[i];
-        sd.R = rad[i];
-        sd.Ns = Ns;
-        sd.ns_shift = log2_or_neg(Ns);
-        sd.nb = L / sd.R;
-        sd.nb_shift = log2_or_neg(sd.nb);
-        sd.ts = L / (Ns * sd.R);
-        Ns *= sd.R;
-    }
-    return p;
-}
-
 // Icosphere: level-L subdivided icosahedron, vertex weights = 1/3 of the
 // adjacent spherical-triangle areas (sum 4 pi).
 bool icosphere(int n_dir, std::vector<double>& dirs, std::vector<double>& wts) {
@@ -397,7 +365,6 @@ void set_grid(eels_ctx* c, const eels_grid* g) {
     L.colinfo = c->colinfo.as<int4>();
     L.contig = contig ? 1 : 0;
     L.nmat = maxm;
-    L.px = make_plan(Mx); L.py = make_plan(My); L.pz = make_plan(Mz);
     L.qx = make_plan2(Mx); L.qy = make_plan2(My); L.qz = make_plan2(Mz);
     L.s32 = make_slab_plan(L, sizeof(float2));
     L.s64 = make_slab_plan(L, sizeof(double2));
@@ -605,6 +572,11 @@ LatticeDev dhat_lattice(eels_ctx* c, int interaction) {
         L.igt = c->igt_tab.as<double>();
     }
     return L;
+}
+
+// Energies whose D-hat is built together: as many as fit `bytes` of scratch.
+int dhat_chunk(const LatticeDev& L, int n_slot, size_t bytes) {
+    return (int)std::max<size_t>(1, std::min<size_t>({(size_t)n_slot, bytes / dhat_scratch_bytes(L), 4096}));
 }
 
 // Iterations allowed per inner solve: an FP32 inner solve may be restarted
@@ -1070,8 +1042,8 @@ int solve_impl(eels_ctx* c, const eels_opts* o, int n_energy, const double* ener
         c->Dr32.ensure((size_t)n_slot * 6 * L.Hx * L.Hy * L.Hz * sizeof(float2));
         c->Dx32.ensure((size_t)n_slot * 6 * L.Hx * L.Hy * L.Hz * sizeof(float2));
         // D-hat for the batch energies, in chunks that fit ~1/8 of the system budget
-        const int gchunk = (int)std::max<size_t>(1, std::min<size_t>(n_slot, (size_t)std::max(1, S) * per_sys / 8 / gslot + 1));
-        c->G.ensure(gchunk * gslot);
+        const int gchunk = dhat_chunk(L, n_slot, (size_t)std::max(1, S) * per_sys / 8 + gslot);
+        c->G.ensure(gchunk * dhat_scratch_bytes(L));
         std::vector<double2> kap_slot(n_slot);
         for (int e = e0; e < e1; ++e) kap_slot[e - e0] = d2(ep[e].kappa);
         h2d(c->kappa_slot, kap_slot, st);
@@ -1466,7 +1438,7 @@ int eels_apply_matrix(eels_ctx* c, int precision, double energy_eV, int n_mat, c
         c->Dr64.ensure(hs * sizeof(double2));
         c->Dr32.ensure(hs * sizeof(float2));
         c->Dx32.ensure(hs * sizeof(float2));
-        c->G.ensure((size_t)6 * L.Mx * L.My * L.Mz * sizeof(double2));
+        c->G.ensure(dhat_scratch_bytes(L));
         std::vector<double2> ks(1, d2(p.kappa));
         h2d(c->kappa_slot, ks, st);
         launch_dhat_build(dhat_lattice(c, c->interaction), 1, c->kappa_slot.as<double2>(), c->G.as<double2>(),
@@ -1534,8 +1506,6 @@ int eels_prepare_operator(eels_ctx* c, int n_energy, const double* energy_eV, in
         c->Dr64.ensure(S * hs * sizeof(double2));
         c->Dr32.ensure(S * hs * sizeof(float2));
         c->Dx32.ensure(S * hs * sizeof(float2));
-        const size_t gslot = (size_t)6 * L.Mx * L.My * L.Mz * sizeof(double2);
-        c->G.ensure(gslot);
         std::vector<double2> kap, coef((size_t)S * EELS_MAX_MAT), diag((size_t)S * EELS_MAX_MAT, make_double2(1, 0));
         std::vector<int> slot(S);
         // consecutive systems with the same energy and permittivities share one
@@ -1555,9 +1525,12 @@ int eels_prepare_operator(eels_ctx* c, int n_energy, const double* energy_eV, in
             for (int m = 0; m < EELS_MAX_MAT; ++m) coef[(size_t)e * EELS_MAX_MAT + m] = m < n_mat ? d2(p.sa[m]) : make_double2(0, 0);
         }
         h2d(c->kappa_slot, kap, st);
-        for (size_t e = 0; e < kap.size(); ++e)
-            launch_dhat_build(dhat_lattice(c, c->interaction), 1, c->kappa_slot.as<double2>() + e, c->G.as<double2>(),
-                              c->Dr64.as<double2>() + e * hs,
+        const int n_slot = (int)kap.size();
+        const int gchunk = dhat_chunk(L, n_slot, (size_t)6 * L.Mx * L.My * L.Mz * sizeof(double2));
+        c->G.ensure(gchunk * dhat_scratch_bytes(L));
+        for (int e = 0; e < n_slot; e += gchunk)
+            launch_dhat_build(dhat_lattice(c, c->interaction), std::min(gchunk, n_slot - e),
+                              c->kappa_slot.as<double2>() + e, c->G.as<double2>(), c->Dr64.as<double2>() + e * hs,
                               c->Dr32.as<float2>() + e * hs, st, c->Dx32.as<float2>() + e * hs);
         c->spb = std::min(max_run, 16);
         h2d(c->coef, coef, st); h2d(c->diag, diag, st); h2d(c->slot, slot, st);

@@ -13,7 +13,7 @@
 // then runs on two inputs.  Twiddles come from a callable tw(k) returning
 // exp(-2 pi i p k / L) for this lane (a shared table or registers).
 #pragma once
-#include "fft.cuh"
+#include "dft.cuh"
 
 namespace eels {
 

@@ -1,4 +1,4 @@
-// FFT kernels of the DDA matrix-vector product and of the D-hat build.
+// FFT kernels of the DDA matrix-vector product.
 //
 // The interaction sum conv(u)_i = sum_{j != i} G~'(r_i - r_j) u_j over a
 // cubic lattice is a 3-D convolution; embedding it in a circulant of
@@ -11,8 +11,8 @@
 // fastest): a slab pass (gather, y and z transforms of one x-slab), the x pass
 // (My*Mz lines: x transform, D-hat product, inverse x transform) and a slab
 // pass back (inverse z and y transforms, combination with x, scatter).  This
-// file holds the slab passes of 64 x 64 and 128 x 128 points in FP32, the D-hat
-// build and the launch of a matvec; k_slab.cuh and k_xline.cuh the passes of
+// file holds the slab passes of 64 x 64 and 128 x 128 points in FP32 and the
+// launch of a matvec; k_dhat.cu the D-hat build, k_slab.cuh and k_xline.cuh the passes of
 // any length, k_xreg.cu the x pass of 64 and 128 points in FP32.
 //
 // D-hat is stored on the octant 0 <= k <= M/2 only (6 (M/2+1)^3 values):
@@ -34,140 +34,6 @@ template <> __device__ __forceinline__ const double2* tw_of<double>(const Lattic
 }
 template <> __device__ __forceinline__ const float2* tw_of<float>(const LatticeDev& L, int axis) {
     return axis == 0 ? L.tw32x : (axis == 1 ? L.tw32y : L.tw32z);
-}
-
-// ---------------------------------------------------------------------------
-// Generic pass along one axis of a batch of arrays [nb][n1][n2][n3].
-// Reads the first in_len entries of every line (zero-extended to the FFT
-// length), writes the first out_len outputs in place.
-// ---------------------------------------------------------------------------
-template <typename Rl, int W, bool INV, int AXIS>
-__global__ void __launch_bounds__(FFT_THREADS) k_axis(cx<Rl>* data, int n1, int n2, int n3, int in_len, int out_len,
-                                                      FftPlan p, const cx<Rl>* twg, const int* active, int per_sys) {
-    using C = cx<Rl>;
-    const int b = blockIdx.z;
-    if (active && !active[b / per_sys]) return;
-    const int Lf = p.L;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* tw = reinterpret_cast<C*>(smem_raw);
-    for (int t = threadIdx.x; t < Lf; t += blockDim.x) tw[t] = twg[t];
-    if (AXIS == 3) {
-        const int ls = Lf + 1;
-        C* A = tw + Lf;
-        C* B = A + W * ls;
-        const int i1 = blockIdx.y, i20 = blockIdx.x * W;
-        C* base = data + ((size_t)b * n1 + i1) * (size_t)n2 * n3;
-        for (int t = threadIdx.x; t < W * Lf; t += blockDim.x) {
-            const int i = t % Lf, w = t / Lf, i2 = i20 + w;
-            A[w * ls + i] = (i < in_len && i2 < n2) ? base[(size_t)i2 * n3 + i] : mk<C>(0.0, 0.0);
-        }
-        __syncthreads();
-        const C* r = fft_lines<INV, false, W>(A, B, ls, 1, p, tw);
-        for (int t = threadIdx.x; t < W * out_len; t += blockDim.x) {
-            const int i = t % out_len, w = t / out_len, i2 = i20 + w;
-            if (i2 < n2) base[(size_t)i2 * n3 + i] = r[w * ls + i];
-        }
-    } else {
-        const int es = W + 1;
-        C* A = tw + Lf;
-        C* B = A + Lf * es;
-        const int fixed = blockIdx.y, i30 = blockIdx.x * W;
-        size_t base, stride;
-        if (AXIS == 1) { base = (size_t)b * n1 * n2 * n3 + (size_t)fixed * n3; stride = (size_t)n2 * n3; }
-        else { base = ((size_t)b * n1 + fixed) * (size_t)n2 * n3; stride = (size_t)n3; }
-        C* d = data + base;
-        for (int t = threadIdx.x; t < W * Lf; t += blockDim.x) {
-            const int w = t % W, i = t / W, i3 = i30 + w;
-            A[i * es + w] = (i < in_len && i3 < n3) ? d[(size_t)i * stride + i3] : mk<C>(0.0, 0.0);
-        }
-        __syncthreads();
-        const C* r = fft_lines<INV, true, W>(A, B, 1, es, p, tw);
-        for (int t = threadIdx.x; t < W * out_len; t += blockDim.x) {
-            const int w = t % W, i = t / W, i3 = i30 + w;
-            if (i3 < n3) d[(size_t)i * stride + i3] = r[i * es + w];
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------
-// D-hat build: G~'(R) on the padded lattice, R in units of d, for n_slot
-// wavenumbers kappa = k d.  Layout G[slot][comp][y][x][z].
-//   G~' = exp(i kappa R)/R [kappa^2 (I - RR) - (1 - i kappa R)/R^2 (I - 3 RR)]   (Eq. 5)
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ int wrap_disp(int i, int n, int m, bool* ok) {
-    if (i < n) return i;
-    if (i > m - n) return i - m;
-    *ok = false;
-    return 0;
-}
-
-__global__ void k_green(LatticeDev L, const double2* kappa, double2* G) {
-    const size_t M = (size_t)L.Mx * L.My * L.Mz;
-    const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= M) return;
-    const int slot = blockIdx.y;
-    const int z = (int)(idx % L.Mz);
-    const int x = (int)((idx / L.Mz) % L.Mx);
-    const int y = (int)(idx / ((size_t)L.Mz * L.Mx));
-    bool ok = true;
-    const double rx = wrap_disp(x, L.Nx, L.Mx, &ok);
-    const double ry = wrap_disp(y, L.Ny, L.My, &ok);
-    const double rz = wrap_disp(z, L.Nz, L.Mz, &ok);
-    double2 g[6];
-    for (int c = 0; c < 6; ++c) g[c] = make_double2(0.0, 0.0);
-    const double rn2 = rx * rx + ry * ry + rz * rz;
-    const bool near = L.igt && fabs(rx) <= IGT_NEAR && fabs(ry) <= IGT_NEAR && fabs(rz) <= IGT_NEAR;
-    if (ok && rn2 > 0.0 && near) {
-        // cell-averaged tensor to second order in kappa: exp(i kappa R)(-T0 + i kappa T1 + kappa^2 T2)
-        const int side = 2 * IGT_NEAR + 1;
-        const double* t = L.igt + ((size_t)(((int)rz + IGT_NEAR) * side + ((int)ry + IGT_NEAR)) * side +
-                                   ((int)rx + IGT_NEAR)) * 18;
-        const double rn = sqrt(rn2);
-        const double2 kap = kappa[slot];
-        double sn, cs;
-        sincos(kap.x * rn, &sn, &cs);
-        const double ex = exp(-kap.y * rn);
-        const double2 ph = make_double2(ex * cs, ex * sn);
-        const double2 ik = make_double2(-kap.y, kap.x);
-        const double2 k2 = kap * kap;
-        for (int c = 0; c < 6; ++c) {
-            const double2 v = make_double2(-t[c], 0.0) + t[6 + c] * ik + t[12 + c] * k2;
-            g[c] = ph * v;
-        }
-    } else if (ok && rn2 > 0.0) {
-        const double rn = sqrt(rn2);
-        const double h[3] = {rx / rn, ry / rn, rz / rn};
-        const double2 kap = kappa[slot];
-        // exp(i kappa R) / R
-        const double2 ikr = make_double2(-kap.y * rn, kap.x * rn);
-        double sn, cs;
-        sincos(ikr.y, &sn, &cs);
-        const double ex = exp(ikr.x) / rn;
-        const double2 ph = make_double2(ex * cs, ex * sn);
-        const double2 k2 = kap * kap;
-        const double2 t = (1.0 / rn2) * make_double2(1.0 - ikr.x, -ikr.y);   // (1 - i kappa R)/R^2
-        const int pa[6] = {0, 0, 0, 1, 1, 2}, pb[6] = {0, 1, 2, 1, 2, 2};
-        for (int c = 0; c < 6; ++c) {
-            const double hh = h[pa[c]] * h[pb[c]];
-            const double dd = pa[c] == pb[c] ? 1.0 : 0.0;
-            g[c] = ph * ((dd - hh) * k2 - (dd - 3.0 * hh) * t);
-        }
-    }
-    double2* out = G + (size_t)slot * 6 * M + ((size_t)y * L.Mx + x) * L.Mz + z;
-    for (int c = 0; c < 6; ++c) out[(size_t)c * M] = g[c];
-}
-
-__global__ void k_extract(LatticeDev L, int n_slot, const double2* G, double2* Dr64, float2* Dr32) {
-    const size_t R = (size_t)L.Hx * L.Hy * L.Hz;
-    const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= R * 6 * n_slot) return;
-    const size_t sc = idx / R;          // slot * 6 + comp
-    const size_t r = idx % R;
-    const int kz = (int)(r % L.Hz), kx = (int)((r / L.Hz) % L.Hx), ky = (int)(r / ((size_t)L.Hz * L.Hx));
-    const size_t M = (size_t)L.Mx * L.My * L.Mz;
-    const double2 v = G[sc * M + ((size_t)ky * L.Mx + kx) * L.Mz + kz];
-    Dr64[idx] = v;
-    Dr32[idx] = to_f(v);
 }
 
 // ---------------------------------------------------------------------------
@@ -414,47 +280,10 @@ __global__ void __launch_bounds__(FFT_THREADS, R == 8 ? 4 : 2) k_slab_inv_r(Latt
 // ---------------------------------------------------------------------------
 // Launchers
 // ---------------------------------------------------------------------------
-static const size_t kSmemCap = 220 * 1024;
-
-template <typename Rl> static size_t smem_axis(int Lf, int W, int axis) {
-    return axis == 3 ? (size_t)(Lf + 2 * W * (Lf + 1)) * sizeof(cx<Rl>) : (size_t)(Lf + 2 * Lf * (W + 1)) * sizeof(cx<Rl>);
-}
-
 template <typename K> static void allow_smem(K kernel) {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemCap);
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
     // these kernels keep their working tiles in shared memory: give it the whole carveout
     cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-}
-
-// Pick the widest tile whose shared memory fits a budget that leaves room
-// for two resident blocks per SM (falling back to one block per SM).
-template <typename F> static int pick_w(F smem_of) {
-    for (int W : {32, 16, 8})
-        if (smem_of(W) <= 110 * 1024) return W;
-    for (int W : {16, 8})
-        if (smem_of(W) <= kSmemCap) return W;
-    return 0;
-}
-
-template <typename Rl, int W, bool INV, int AXIS>
-static void axis_launch_w(cx<Rl>* data, int nb, int n1, int n2, int n3, int in_len, int out_len, const FftPlan& p,
-                          const cx<Rl>* tw, const int* active, int per_sys, cudaStream_t st) {
-    dim3 grid;
-    if (AXIS == 3) grid = dim3((n2 + W - 1) / W, n1, nb);
-    else if (AXIS == 1) grid = dim3((n3 + W - 1) / W, n2, nb);
-    else grid = dim3((n3 + W - 1) / W, n1, nb);
-    count_launch();
-    k_axis<Rl, W, INV, AXIS><<<grid, FFT_THREADS, smem_axis<Rl>(p.L, W, AXIS), st>>>(data, n1, n2, n3, in_len, out_len, p, tw,
-                                                                                    active, per_sys);
-}
-
-template <typename Rl, bool INV, int AXIS>
-static void axis_launch(cx<Rl>* data, int nb, int n1, int n2, int n3, int in_len, int out_len, const FftPlan& p,
-                        const cx<Rl>* tw, const int* active, int per_sys, cudaStream_t st) {
-    const int W = pick_w([&](int w) { return smem_axis<Rl>(p.L, w, AXIS); });
-    if (W == 32) axis_launch_w<Rl, 32, INV, AXIS>(data, nb, n1, n2, n3, in_len, out_len, p, tw, active, per_sys, st);
-    else if (W == 16) axis_launch_w<Rl, 16, INV, AXIS>(data, nb, n1, n2, n3, in_len, out_len, p, tw, active, per_sys, st);
-    else axis_launch_w<Rl, 8, INV, AXIS>(data, nb, n1, n2, n3, in_len, out_len, p, tw, active, per_sys, st);
 }
 
 // Register-resident slab kernels: FP32 with 64- or 128-point y and z transforms.
@@ -562,18 +391,10 @@ void launch_matvec(const LatticeDev& L, const MatvecArgs<Rl>& a, cudaStream_t st
     slab_launch_any<Rl>(L, a, true, st);
 }
 
-template <typename Rl, int W> static void prepare_w() {
-    allow_smem(k_axis<Rl, W, false, 1>);
-    allow_smem(k_axis<Rl, W, false, 2>);
-    allow_smem(k_axis<Rl, W, false, 3>);
-}
-
 void prepare_far_kernels();
 void prepare_xreg_kernels();
 
 void prepare_kernels() {
-    prepare_w<float, 8>(); prepare_w<float, 16>(); prepare_w<float, 32>();
-    prepare_w<double, 8>(); prepare_w<double, 16>(); prepare_w<double, 32>();
     allow_smem(k_slab_fwd_r<8, true, true>);
     allow_smem(k_slab_fwd_r<8, true, false>);
     allow_smem(k_slab_fwd_r<8, false, true>);
@@ -604,22 +425,6 @@ template void launch_matvec<double>(const LatticeDev&, const MatvecArgs<double>&
 static bool slab_reg(const LatticeDev& L) { return (L.My == 64 && L.Mz == 64) || (L.My == 128 && L.Mz == 128); }
 int matvec_dot_parts(const LatticeDev& L, bool fp64) {
     return 3 * L.Nx * (fp64 ? L.s64.CL : slab_reg(L) ? 1 : L.s32.CL);
-}
-
-void launch_dhat_build(const LatticeDev& L, int n_slot, const double2* kappa, double2* G, double2* Dr64, float2* Dr32,
-                       cudaStream_t st, float2* Dx32) {
-    const size_t M = (size_t)L.Mx * L.My * L.Mz;
-    dim3 g1((unsigned)((M + 255) / 256), n_slot);
-    count_launch();
-    k_green<<<g1, 256, 0, st>>>(L, kappa, G);
-    const int nb = n_slot * 6;
-    axis_launch<double, false, 3>(G, nb, L.My, L.Mx, L.Mz, L.Mz, L.Mz, L.pz, L.tw64z, nullptr, 1, st);
-    axis_launch<double, false, 1>(G, nb, L.My, L.Mx, L.Mz, L.My, L.My, L.py, L.tw64y, nullptr, 1, st);
-    axis_launch<double, false, 2>(G, nb, L.My, L.Mx, L.Mz, L.Mx, L.Mx, L.px, L.tw64x, nullptr, 1, st);
-    const size_t R = (size_t)L.Hx * L.Hy * L.Hz * 6 * n_slot;
-    count_launch();
-    k_extract<<<(unsigned)((R + 255) / 256), 256, 0, st>>>(L, n_slot, G, Dr64, Dr32);
-    if (Dx32) launch_dhat_interleave(L, n_slot, Dr64, Dx32, st);
 }
 
 }  // namespace eels

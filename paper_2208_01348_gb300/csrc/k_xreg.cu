@@ -521,23 +521,6 @@ k_xpass_tma(LatticeDev L, MatvecArgs<float> a, const __grid_constant__ CUtensorM
     }
 }
 
-// FP32 copy of the octant D-hat for the register x pass:
-// Dx[slot][ky][kz][comp][kx] from Dr64[slot][comp][ky][kx][kz].
-__global__ void k_dhat_interleave(LatticeDev L, int n_slot, const double2* __restrict__ Dr64, float2* __restrict__ Dx) {
-    const size_t R = (size_t)L.Hx * L.Hy * L.Hz;
-    const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= R * 6 * n_slot) return;
-    const int kx = (int)(idx % L.Hx);
-    const size_t t = idx / L.Hx;                     // ((slot * Hy + ky) * Hz + kz) * 6 + comp
-    const int comp = (int)(t % 6);
-    const int kz = (int)((t / 6) % L.Hz);
-    const size_t sy = t / (6 * (size_t)L.Hz);        // slot * Hy + ky
-    const int ky = (int)(sy % L.Hy);
-    const size_t slot = sy / L.Hy;
-    const double2 v = Dr64[((slot * 6 + comp) * L.Hy + ky) * (size_t)L.Hx * L.Hz + (size_t)kx * L.Hz + kz];
-    Dx[idx] = to_f(v);
-}
-
 bool xpass_reg_supported(const LatticeDev& L) {
     return (L.Mx == 64 || L.Mx == 128) && 2 * L.Nx <= L.Mx && L.Mz % 2 == 0;
 }
@@ -669,12 +652,6 @@ unsigned int wait_timeouts() {
         return 0;
     }
     return v;
-}
-
-void launch_dhat_interleave(const LatticeDev& L, int n_slot, const double2* Dr64, float2* Dx, cudaStream_t st) {
-    const size_t n = (size_t)L.Hx * L.Hy * L.Hz * 6 * n_slot;
-    count_launch();
-    k_dhat_interleave<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(L, n_slot, Dr64, Dx);
 }
 
 }  // namespace eels

@@ -9,7 +9,6 @@
 
 #include "common.cuh"
 #include "dft.cuh"
-#include "fft.cuh"
 
 namespace eels {
 
@@ -47,7 +46,6 @@ struct LatticeDev {
     int nmat;                     // materials used by the lattice (1: one coefficient per system)
     const double* igt;            // D-hat build only: cell tables of the igt_so interaction (igt.cu), or
                                   // nullptr for point dipoles
-    FftPlan px, py, pz;
     Plan2 qx, qy, qz;
     SlabPlan s32, s64;            // slab passes in FP32 and FP64
     int xw32, xw64;               // x-pass tile width chosen by the autotuner (0: size heuristic)
@@ -102,13 +100,13 @@ int matvec_dot_parts(const LatticeDev& L, bool fp64);
 template <typename Rl>
 void launch_matvec(const LatticeDev& L, const MatvecArgs<Rl>& a, cudaStream_t st);
 
-// D-hat build for n_slot energies: kappa[slot] = k d (complex).  G scratch
-// [n_slot][6][My][Mx][Mz] FP64; outputs reduced D-hat FP64 and FP32.
-void launch_dhat_build(const LatticeDev& L, int n_slot, const double2* kappa, double2* Gscratch,
-                       double2* Dr64, float2* Dr32, cudaStream_t st, float2* Dx32 = nullptr);
-// FP32 copy Dx[slot][ky][kz][comp][kx] of the octant D-hat (read by the
+// D-hat build for n_slot energies: kappa[slot] = k d (complex).  Scratch of
+// n_slot * dhat_scratch_bytes; outputs the octant D-hat [slot][comp][ky][kx][kz]
+// in FP64 and FP32 and, with Dx32, [slot][ky][kz][comp][kx] (read by the
 // register-resident x pass).
-void launch_dhat_interleave(const LatticeDev& L, int n_slot, const double2* Dr64, float2* Dx, cudaStream_t st);
+size_t dhat_scratch_bytes(const LatticeDev& L);
+void launch_dhat_build(const LatticeDev& L, int n_slot, const double2* kappa, double2* scratch,
+                       double2* Dr64, float2* Dr32, cudaStream_t st, float2* Dx32 = nullptr);
 // Register-resident x pass (Mx = 64 or 128, FP32): false when the lattice or
 // the arguments do not suit it (the caller then launches the shared-memory one).
 bool xpass_reg_supported(const LatticeDev& L);
