@@ -5,6 +5,7 @@
 // register-resident kernels of k_fft.cu instead.
 #pragma once
 #include <cooperative_groups.h>
+#include <cuda_pipeline.h>
 
 #include <algorithm>
 
@@ -41,26 +42,31 @@ template <typename Rl> struct SlabSmem {
         T = S + (size_t)L.My * p.sls;
     }
 };
+// Tables of a block, copied asynchronously in two groups: the column table, then
+// the twiddles.
 template <typename Rl>
 __device__ __forceinline__ void slab_tables(const LatticeDev& L, const MatvecArgs<Rl>& a, const SlabSmem<Rl>& m, int s,
                                             int ix) {
     using C = cx<Rl>;
+    if (L.contig)
+        for (int t = threadIdx.x; t < L.Ny; t += blockDim.x)
+            __pipeline_memcpy_async(m.ci + t, L.colinfo + (size_t)ix * L.Ny + t, sizeof(int4));
+    __pipeline_commit();
     const C* gy = slab_tw<Rl>(L, 1);
     const C* gz = slab_tw<Rl>(L, 2);
     for (int t = threadIdx.x; t < L.My; t += blockDim.x) {
         const int r = (int)L.qy.dRe.div(t), j = t - r * L.qy.Re;
-        m.twy[t] = gy[r * j];
+        __pipeline_memcpy_async(m.twy + t, gy + r * j, sizeof(C));
     }
     for (int t = threadIdx.x; t < L.Mz; t += blockDim.x) {
         const int r = (int)L.qz.dRe.div(t), j = t - r * L.qz.Re;
-        m.twz[t] = gz[r * j];
+        __pipeline_memcpy_async(m.twz + t, gz + r * j, sizeof(C));
     }
+    __pipeline_commit();
     if (threadIdx.x < EELS_MAX_MAT) {
         m.cf[threadIdx.x] = cvt<C>(a.coef[(size_t)s * EELS_MAX_MAT + threadIdx.x]);
         m.dg[threadIdx.x] = cvt<C>(a.diag[(size_t)s * EELS_MAX_MAT + threadIdx.x]);
     }
-    if (L.contig)
-        for (int t = threadIdx.x; t < L.Ny; t += blockDim.x) m.ci[t] = L.colinfo[(size_t)ix * L.Ny + t];
 }
 
 template <typename Rl, bool CLUSTER>
@@ -73,6 +79,7 @@ __global__ void __launch_bounds__(sizeof(Rl) == 4 ? 768 : 512, 1) k_slab_fwd(Lat
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const SlabSmem<Rl> m(smem_raw, L, sp);
     slab_tables<Rl>(L, a, m, s, ix);
+    __pipeline_wait_prior(1);
     __syncthreads();
     const int Ny = L.Ny, Nz = L.Nz;
     SlabCtx<Rl> sc;
@@ -96,6 +103,7 @@ __global__ void __launch_bounds__(sizeof(Rl) == 4 ? 768 : 512, 1) k_slab_fwd(Lat
 #define Y1(R) case R: slab_y1<R, Rl>(sc, ry, dcol, Ny, threadIdx.x, blockDim.x, gather); break;
         EELS_SWITCH_RE(L.qy.Re, Y1)
 #undef Y1
+        __pipeline_wait_prior(0);
         __syncthreads();
 #define YM(R) case R: slab_ymid<R, false, Rl>(sc, ry, dcol, threadIdx.x, blockDim.x); break;
         EELS_SWITCH_RO(L.qy.Ro, YM)
@@ -104,6 +112,7 @@ __global__ void __launch_bounds__(sizeof(Rl) == 4 ? 768 : 512, 1) k_slab_fwd(Lat
 #define Y(RE, RO)                                                                                     \
     case RE * RO:                                                                                     \
         slab_y1<RE, Rl>(sc, CtPlan<RE, RO>{}, dcol, Ny, threadIdx.x, blockDim.x, gather);             \
+        __pipeline_wait_prior(0);                                                                     \
         __syncthreads();                                                                              \
         slab_ymid<RO, false, Rl>(sc, CtPlan<RE, RO>{}, dcol, threadIdx.x, blockDim.x);                \
         break;
@@ -161,6 +170,7 @@ __global__ void __launch_bounds__(sizeof(Rl) == 4 ? 768 : 512, 1) k_slab_inv(Lat
     __shared__ Rl red[2 * 24];
     const SlabSmem<Rl> m(smem_raw, L, sp);
     slab_tables<Rl>(L, a, m, s, ix);
+    __pipeline_wait_prior(0);
     if (CLUSTER) cg::this_cluster().sync();           // every block of the cluster runs before the remote stores
     else __syncthreads();
     const int Ny = L.Ny, Nz = L.Nz;
