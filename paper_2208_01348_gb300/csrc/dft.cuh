@@ -153,11 +153,10 @@ template <bool INV, typename C> struct Dft<3, INV, C> {
         using Rl = decltype(v[0].x);
         const Rl c = (Rl)K_C3, s = (Rl)(INV ? -K_S3 : K_S3);
         C a = v[1] + v[2], b = v[1] - v[2];
-        C m = v[0] + c * a;
-        C jb; jb.x = s * b.y; jb.y = -s * b.x;   // -i s b
+        const C m = fma_s(c, a, v[0]), jb = mul_mi(b);   // +- s (-i b)
         v[0] = v[0] + a;
-        v[1] = m + jb;
-        v[2] = m - jb;
+        v[1] = fma_s(s, jb, m);
+        v[2] = fma_s(-s, jb, m);
     }
 };
 template <bool INV, typename C> struct Dft<4, INV, C> {
@@ -176,20 +175,20 @@ template <bool INV, typename C> struct Dft<8, INV, C> {
         C o[4] = {v[1], v[3], v[5], v[7]};
         Dft<4, INV, C>::run(e);
         Dft<4, INV, C>::run(o);
-        // twiddles exp(-+ 2 pi i p / 8), p = 1, 2, 3
-        C t1, t3;
+        // twiddles exp(-+ 2 pi i p / 8), p = 1, 2, 3: h (1 -+ i), -+i, -h (1 +- i)
+        C w1, w3;
         if (!INV) {
-            t1.x = h * (o[1].x + o[1].y); t1.y = h * (o[1].y - o[1].x);
-            t3.x = h * (o[3].y - o[3].x); t3.y = -h * (o[3].x + o[3].y);
+            w1.x = o[1].x + o[1].y; w1.y = o[1].y - o[1].x;
+            w3.x = o[3].y - o[3].x; w3.y = -o[3].x - o[3].y;
         } else {
-            t1.x = h * (o[1].x - o[1].y); t1.y = h * (o[1].y + o[1].x);
-            t3.x = -h * (o[3].x + o[3].y); t3.y = h * (o[3].x - o[3].y);
+            w1.x = o[1].x - o[1].y; w1.y = o[1].y + o[1].x;
+            w3.x = -o[3].x - o[3].y; w3.y = o[3].x - o[3].y;
         }
-        C t2 = rot_mi<INV>(o[2]);
+        const C t2 = rot_mi<INV>(o[2]);
         v[0] = e[0] + o[0]; v[4] = e[0] - o[0];
-        v[1] = e[1] + t1;   v[5] = e[1] - t1;
+        v[1] = fma_s(h, w1, e[1]); v[5] = fma_s(-h, w1, e[1]);
         v[2] = e[2] + t2;   v[6] = e[2] - t2;
-        v[3] = e[3] + t3;   v[7] = e[3] - t3;
+        v[3] = fma_s(h, w3, e[3]); v[7] = fma_s(-h, w3, e[3]);
     }
 };
 
@@ -209,11 +208,11 @@ template <int R, bool INV, typename C> struct DftOdd {
         v[0] = x0;
 #pragma unroll
         for (int p = 1; p <= H; ++p) {
-            C re = v0 + (Rl)cs[p] * sp[0], im = (Rl)sn[p] * sm[0];
+            C re = fma_s((Rl)cs[p], sp[0], v0), im = (Rl)sn[p] * sm[0];
 #pragma unroll
             for (int q = 2; q <= H; ++q) {
-                re = re + (Rl)cs[(p * q) % R] * sp[q - 1];
-                im = im + (Rl)sn[(p * q) % R] * sm[q - 1];
+                re = fma_s((Rl)cs[(p * q) % R], sp[q - 1], re);
+                im = fma_s((Rl)sn[(p * q) % R], sm[q - 1], im);
             }
             const C jim = INV ? mul_i(im) : mul_mi(im);   // forward: -i im; inverse: +i im
             v[p] = re + jim;
