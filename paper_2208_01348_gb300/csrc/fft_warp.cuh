@@ -17,12 +17,12 @@
 
 namespace eels {
 
-constexpr int R64_QS = 132;   // transpose tile strides (8-byte units): line -> 4, lane -> 1 (mod 16)
-constexpr int R64_PS = 17;
-constexpr int R64_TILE = 4 * R64_QS;
-constexpr int R128_QS = 148;  // transpose tile strides (8-byte units): line -> 4, lane -> 1 (mod 16)
-constexpr int R128_PS = 17;
-constexpr int R128_TILE = 4 * R128_QS;
+// Transpose tile strides (8-byte units), even and line -> 4 (mod 16): a lane
+// writes its row in 16-byte pieces (half the instructions of 8-byte stores at
+// the same wavefronts), and the 8 lanes of each quarter-warp store as well as
+// the 16 of each half-warp load fall on distinct banks.
+constexpr int R64_QS = 84, R64_PS = 10, R64_TILE = 4 * R64_QS;
+constexpr int R128_QS = 148, R128_PS = 17, R128_TILE = 4 * R128_QS;
 
 // Length-4 DFT of (a, b, 0, 0): out = (a + b, a + rot(b), a - b, a - rot(b)),
 // rot = multiplication by -i (forward) or +i (inverse).
@@ -110,7 +110,8 @@ __device__ __forceinline__ void fft64_warp_t(float2 (&v)[8], float2* tile, int q
         v[k] = v[k] * w;
     }
 #pragma unroll
-    for (int k = 0; k < 8; ++k) tile[q * R64_QS + p * R64_PS + k] = v[k];
+    for (int k = 0; k < 8; k += 2)
+        *reinterpret_cast<float4*>(tile + q * R64_QS + p * R64_PS + k) = make_float4(v[k].x, v[k].y, v[k + 1].x, v[k + 1].y);
     __syncwarp();
 #pragma unroll
     for (int i = 0; i < 8; ++i) v[i] = tile[q * R64_QS + i * R64_PS + p];

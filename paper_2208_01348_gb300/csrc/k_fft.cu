@@ -62,7 +62,7 @@ template <int R> struct SlabRSmem {
     float2 tw2[(R - 1) * 8];                     // exp(-2 pi i p k / L) at [k - 1][p]: conflict-free per k
     float2 cf[EELS_MAX_MAT], dg[EELS_MAX_MAT];   // this system's per-material coefficients
     float2 S[SlabR<R>::L * SlabR<R>::SLS];
-    float2 tile[FFT_THREADS / 32][SlabR<R>::TILE];
+    alignas(16) float2 tile[FFT_THREADS / 32][SlabR<R>::TILE];
     int4 ci[SlabR<R>::L / 2];                    // this slab's column table (contiguous columns)
 };
 

@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(XR_THREADS, 4) k_xpass_reg(LatticeDev L, Matve
     constexpr int ZT = X::ZT;
     __shared__ float2 tws[MX];                          // exp(-2 pi i t / MX)
     __shared__ float2 tw2[7 * 8];                       // w64^(p k) at [k - 1][p]: lanes p read consecutive words
-    __shared__ float2 tiles[XR_WARPS][R64_TILE];
+    __shared__ __align__(16) float2 tiles[XR_WARPS][R64_TILE];
     __shared__ __align__(16) float2 dt[(ZT + 1) * X::RS];
     __shared__ __align__(8) unsigned long long bar;
     const int kyr = blockIdx.y, z0 = blockIdx.x * ZT;
@@ -285,17 +285,27 @@ __global__ void __launch_bounds__(XR_THREADS, 4) k_xpass_reg(LatticeDev L, Matve
 // ---------------------------------------------------------------------------
 // The same x pass with the U lines moved by the tensor memory accelerator.
 //
-// When Mz is a multiple of 2 ZT, the kz lines pair into aligned tiles: the
+// PAIR (Mz a multiple of 2 ZT): the kz lines pair into aligned tiles: the
 // direct tile kz in [z0, z0 + ZT) (kz' = kz) and the mirror tile
 // kz in [Mz - z0 - ZT, Mz - z0) (kz' = Mz - kz in (z0, z0 + ZT]); both use
 // the D-hat rows kz' in [z0, z0 + ZT], and every kz (kz = Mz/2 included, in
-// the mirror tile of the last z0) belongs to exactly one tile.  A pass moves
+// the mirror tile of the last z0) belongs to exactly one tile.  Otherwise the
+// tiles [z0, z0 + ZT) cover all of [0, Mz), each with its own D-hat rows; the
+// copies fill and clip what a tile has past Mz.  A pass moves
 // the three components of one tile, Nx rows x ZT kz each, into shared memory
 // with one 4-D tensor copy (box ZT x Nx x 1 x 3 of U viewed as
 // [3S][My][Nx][Mz]), transforms it in registers as k_xpass_reg does, writes
 // the results back into the same buffer (each warp owns its columns) and
 // stores the tile with one tensor copy; two buffers let the copy of the next
 // pass overlap the current one.
+//
+// What bounds it: the LSU's data pipe (shared-memory wavefronts, 76 % of its
+// rate at 128 points, 83 % at 64 with packed additions).  Hence the 16-byte
+// exchange stores, the twiddles in registers and, at 64 points, the column and
+// D-hat row maps that keep the swizzled tile's accesses off each other's banks:
+// 95 -> 78 M wavefronts and 375 -> 338 us for 200 systems of 64^3 points, 417 ->
+// 409 us for 25 of 128^3.  The rod (Mz = 144, lone tiles): 0.97 -> 0.70 ms for
+// 256 beams, against k_xpass_reg whose loads meet 8 rows each.
 // ---------------------------------------------------------------------------
 template <int MX> struct XTma {
     static constexpr int ZT = XReg<MX>::ZT;
@@ -313,7 +323,7 @@ template <int MX> struct XTma {
 template <int MX> struct XTmaSmem {
     float2 ut[2][XTma<MX>::TILE];                       // U tiles (tensor-copy destinations, 1024-byte aligned)
     float2 dt[(XReg<MX>::ZT + 1) * XReg<MX>::RS];      // D-hat rows kz' in [z0, z0 + ZT]
-    float2 tiles[XR_WARPS][R64_TILE];                   // warp-private transposes
+    alignas(16) float2 tiles[XR_WARPS][R64_TILE];       // warp-private transposes
     float2 tws[MX];
     float2 tw2[7 * 8];
     unsigned long long bar_d, bar_u[2];
@@ -323,7 +333,15 @@ struct XPass {
     int s, ky, mirror;
 };
 
-template <int MX>
+// Place of D-hat row r (kz' minus the block's first row) in shared memory: with
+// Mx = 64 a warp's columns are {2w, 2w + 1, 2w + 8, 2w + 9}, whose rows (in
+// either direction) differ in bits 0 and 3; they go to places that differ in
+// bits 0 and 1, so that rows of RS = 4 (mod 16) words meet four bank groups.
+template <int MX> __device__ __forceinline__ int drow_place(int r) {
+    return MX == 64 ? (r & 16) | ((r >> 1 & 3) << 2) | (r >> 3 & 1) << 1 | (r & 1) : r;
+}
+
+template <int MX, bool PAIR>
 __global__ void __launch_bounds__(XR_THREADS, 3)
 k_xpass_tma(LatticeDev L, MatvecArgs<float> a, const __grid_constant__ CUtensorMap umap) {
     using X = XReg<MX>;
@@ -346,7 +364,10 @@ k_xpass_tma(LatticeDev L, MatvecArgs<float> a, const __grid_constant__ CUtensorM
     const int s_begin = blockIdx.z * a.spb, s_end = min(a.S, s_begin + a.spb);
     const size_t row = (size_t)6 * Hx;
     const int nky = (kyr == 0 || 2 * kyr == My) ? 1 : 2;
-    const int per_sys = 2 * nky;                        // passes per system: ky choices x {direct, mirror}
+    const int per_sys = PAIR ? 2 * nky : nky;           // passes per system: ky choices (x {direct, mirror})
+    const int zl = min(z0 + ZT, Mz) - 1;                // last kz of a lone tile, and the D-hat rows it needs
+    const int row0 = PAIR ? z0 : z0 > Mz / 2 ? Mz - zl : zl > Mz / 2 ? min(z0, Mz - zl) : z0;
+    const int nrow = PAIR ? ZT + 1 : (z0 > Mz / 2 ? Mz - z0 : min(Mz / 2, zl)) - row0 + 1;
     const unsigned tile_bytes = (unsigned)(3 * Nx * ZT * sizeof(float2));
     // pass i of the block: its system (skipping inactive ones), ky and tile
     auto pass_of = [&](int i, XPass& ps) -> bool {
@@ -358,8 +379,8 @@ k_xpass_tma(LatticeDev L, MatvecArgs<float> a, const __grid_constant__ CUtensorM
         }
         if (s >= s_end) return false;
         ps.s = s;
-        ps.ky = (k >> 1) ? My - kyr : kyr;
-        ps.mirror = k & 1;
+        ps.ky = (PAIR ? k >> 1 : k) ? My - kyr : kyr;
+        ps.mirror = PAIR && (k & 1);
         return true;
     };
     auto issue_load = [&](const XPass& ps, int b) {
@@ -382,9 +403,12 @@ k_xpass_tma(LatticeDev L, MatvecArgs<float> a, const __grid_constant__ CUtensorM
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = lane & 3, p = lane >> 2;
     const int h = SPLIT ? (q >> 1) : 0;
-    const int j = warp * X::LPW + (SPLIT ? (q & 1) : q);   // this lane's column of the tile
+    const int j = warp * 2 + (q & 1) + (SPLIT ? 0 : (q >> 1) << 3);   // this lane's column of the tile
     float2* tile = tiles[warp];
-    auto tw = [&](int k) { return tw2[(k - 1) * 8 + p]; };
+    float2 twr[7];                                      // w64^(p k): every transform of the block uses them
+#pragma unroll
+    for (int k = 0; k < 7; ++k) twr[k] = tw2[k * 8 + p];
+    auto tw = [&](int k) { return twr[k - 1]; };
     const float2 zero = make_float2(0.f, 0.f);
     constexpr int RIN = SPLIT ? 8 : 4;
     // element of (component c, row ix, this lane's column j) in a U tile
@@ -405,10 +429,10 @@ k_xpass_tma(LatticeDev L, MatvecArgs<float> a, const __grid_constant__ CUtensorM
             __syncthreads();                             // every thread is done with the previous tile
             if (threadIdx.x == 0) {
                 fence_async_shared();
-                const float2* src = a.Dx + (((size_t)slot * L.Hy + kyr) * L.Hz + z0) * row;
+                const float2* src = a.Dx + (((size_t)slot * L.Hy + kyr) * L.Hz + row0) * row;
                 const unsigned rb = (unsigned)(row * sizeof(float2));
-                mbar_expect_tx(&bar_d, rb * (ZT + 1));
-                for (int r = 0; r <= ZT; ++r) bulk_g2s(dt + r * X::RS, src + r * row, rb, &bar_d);
+                mbar_expect_tx(&bar_d, rb * nrow);
+                for (int r = 0; r < nrow; ++r) bulk_g2s(dt + drow_place<MX>(r) * X::RS, src + r * row, rb, &bar_d);
             }
             // the block decides together, so that no warp leaves while others wait at a barrier
             if (__syncthreads_or(!mbar_wait(&bar_d, ph_d, XR_WAIT_POLLS))) { failed = true; break; }
@@ -427,10 +451,12 @@ k_xpass_tma(LatticeDev L, MatvecArgs<float> a, const __grid_constant__ CUtensorM
         ph_u[b] ^= 1u;
 
         const bool mirror = cur.mirror;
-        const int drow = mirror ? ZT - j : j;           // kz' - z0
-        const bool nyq = mirror && z0 + ZT == Mz / 2 && j == 0;   // kz = Mz/2
+        // kz' - row0; past Mz any row serves (the results are clipped).  At kz = Mz/2 the components odd in z
+        // vanish, so their sign does not matter
+        const int kz = z0 + j;
+        const int drow = PAIR ? (mirror ? ZT - j : j) : kz >= Mz ? 0 : (kz > Mz / 2 ? Mz - kz : kz) - row0;
         const float sy = cur.ky == kyr ? 1.f : -1.f;
-        const float sz = (mirror && !nyq) ? -1.f : 1.f, syz = sy * sz;
+        const float sz = (PAIR ? mirror : kz > Mz / 2) ? -1.f : 1.f, syz = sy * sz;
         float2* T = ut[b];
         float2 v[3][8];
 #pragma unroll
@@ -450,7 +476,7 @@ k_xpass_tma(LatticeDev L, MatvecArgs<float> a, const __grid_constant__ CUtensorM
         }
 #pragma unroll
         for (int c = 0; c < 3; ++c) fft64_warp_t<false, !SPLIT>(v[c], tile, q, p, tw);
-        const float2* Dk = dt + drow * X::RS;
+        const float2* Dk = dt + drow_place<MX>(drow) * X::RS;
 #pragma unroll
         for (int m = 0; m < 8; ++m) {
             const int kx = SPLIT ? 2 * (p + 8 * m) + h : p + 8 * m;
@@ -568,22 +594,28 @@ bool u_tensor_map(const LatticeDev& L, const MatvecArgs<float>& a, int zt, CUten
 template <int MX>
 bool launch_tma(const LatticeDev& L, const MatvecArgs<float>& a, int spb, unsigned groups, cudaStream_t st) {
     constexpr int ZT = XReg<MX>::ZT;
-    if (L.Mz % (2 * ZT) != 0 || ((uintptr_t)a.U & 15) != 0) return false;
+    if (L.Mz < ZT || ((uintptr_t)a.U & 15) != 0) return false;
     CUtensorMap map;
     if (!u_tensor_map(L, a, ZT, &map)) return false;
     MatvecArgs<float> b = a;
     b.spb = spb;
     count_launch();
-    k_xpass_tma<MX><<<dim3(L.Mz / 2 / ZT, L.Hy, groups), XR_THREADS, sizeof(XTmaSmem<MX>) + 1024, st>>>(L, b, map);
+    const size_t sm = sizeof(XTmaSmem<MX>) + 1024;
+    if (L.Mz % (2 * ZT) == 0)
+        k_xpass_tma<MX, true><<<dim3(L.Mz / 2 / ZT, L.Hy, groups), XR_THREADS, sm, st>>>(L, b, map);
+    else
+        k_xpass_tma<MX, false><<<dim3((L.Mz + ZT - 1) / ZT, L.Hy, groups), XR_THREADS, sm, st>>>(L, b, map);
     return true;
 }
 
 }  // namespace
 
 void prepare_xreg_kernels() {
-    cudaFuncSetAttribute(k_xpass_tma<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(XTmaSmem<64>) + 1024);
-    cudaFuncSetAttribute(k_xpass_tma<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)sizeof(XTmaSmem<128>) + 1024);
+    const int s64 = (int)sizeof(XTmaSmem<64>) + 1024, s128 = (int)sizeof(XTmaSmem<128>) + 1024;
+    cudaFuncSetAttribute(k_xpass_tma<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, s64);
+    cudaFuncSetAttribute(k_xpass_tma<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, s64);
+    cudaFuncSetAttribute(k_xpass_tma<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, s128);
+    cudaFuncSetAttribute(k_xpass_tma<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, s128);
 }
 
 bool launch_xpass_reg(const LatticeDev& L, const MatvecArgs<float>& a, cudaStream_t st) {
@@ -626,7 +658,7 @@ void autotune_xreg(const LatticeDev& L, const MatvecArgs<float>& a, int max_spb,
                 CUtensorMap map;
                 constexpr int zt64 = XReg<64>::ZT, zt128 = XReg<128>::ZT;
                 const int zt = L.Mx == 64 ? zt64 : zt128;
-                if (L.Mz % (2 * zt) != 0 || !u_tensor_map(L, a, zt, &map)) break;
+                if (L.Mz < zt || ((uintptr_t)a.U & 15) != 0 || !u_tensor_map(L, a, zt, &map)) break;
             }
             launch_xpass_reg(Lc, ac, st);                // warm-up
             cudaEventRecord(e0, st);
