@@ -69,7 +69,7 @@ TRAFFIC_WORKLOAD = "cherenkov"
 
 def kernel_src_hash() -> str:
     h = hashlib.sha256()
-    for f in ("k_fft.cu", "k_xreg.cu", "fft.cuh", "fft_warp.cuh", "kernels.h", "common.cuh"):
+    for f in ("k_fft.cu", "k_xreg.cu", "dft.cuh", "fft_warp.cuh", "kernels.h", "common.cuh"):
         with open(os.path.join(ROOT, "paper_2208_01348_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
