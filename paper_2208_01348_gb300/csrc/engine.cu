@@ -554,7 +554,7 @@ size_t per_system_bytes(const LatticeDev& L, bool fp64) {
     const size_t vec64 = n3 * sizeof(double2);
     const size_t kvec = n3 * (fp64 ? sizeof(double2) : sizeof(float2));
     const size_t u = (size_t)3 * L.My * L.Nx * L.Mz * sizeof(double2);
-    const int nblk = (int)((n3 + RED_CHUNK - 1) / RED_CHUNK);
+    const int nblk = red_blocks((int)n3, true);       // the more of the two precisions
     return 6 * vec64 + n3 * sizeof(float2) + u + 7 * kvec + 2 * (size_t)nblk * 4 * sizeof(double) + 1024;
 }
 
@@ -596,7 +596,7 @@ KrylovArgs<Rl> krylov_args(eels_ctx* c, int S, const eels_opts* o, double eps) {
     const int n3 = 3 * c->N;
     k.S = S;
     k.n3 = n3;
-    k.nblk = (n3 + RED_CHUNK - 1) / RED_CHUNK;
+    k.nblk = red_blocks(n3, sizeof(Rl) == 8);
     k.nblk_a = k.nblk;
     k.V[0] = c->kv[0].as<cx<Rl>>(); k.V[1] = c->kv[1].as<cx<Rl>>();
     k.P[0] = c->kv[2].as<cx<Rl>>(); k.P[1] = c->kv[3].as<cx<Rl>>(); k.P[2] = c->kv[4].as<cx<Rl>>();
@@ -781,7 +781,7 @@ int refine_rounds(eels_ctx* c, int S, const eels_opts* o, int max_rounds, std::v
                   std::vector<int>& refin) {
     cudaStream_t st = c->stream;
     const int n3 = 3 * c->N;
-    const int nblk = (n3 + RED_CHUNK - 1) / RED_CHUNK;
+    const int nblk = red_blocks(n3, true);
     int* n_outer = c->counters.as<int>() + 1;
     // inner tolerance per system: an FP32 solve is asked for eps_inner (or
     // what the next round still needs, if that is less demanding); an FP64
@@ -904,7 +904,7 @@ void krylov_dev(eels_ctx* c, int solver, const void* b, void* x, int S, double e
                 int* iters, cudaStream_t caller) {
     cudaStream_t st = c->stream;
     const int n3 = 3 * c->N;
-    const int nblk = (n3 + RED_CHUNK - 1) / RED_CHUNK;
+    const int nblk = red_blocks(n3, true);
     const size_t kvec = (size_t)S * n3 * sizeof(cx<Rl>);
     for (auto& v : c->kv) v.ensure(kvec);
     c->part_a.ensure((size_t)S * std::max(nblk, dot_parts(c->L)) * 4 * sizeof(double));
@@ -1023,7 +1023,7 @@ int solve_impl(eels_ctx* c, const eels_opts* o, int n_energy, const double* ener
         const int e0 = s0 / n_beam, e1 = (s0 + S - 1) / n_beam + 1;
         const int n_slot = e1 - e0;
         const int n3 = 3 * c->N;
-        const int nblk = (n3 + RED_CHUNK - 1) / RED_CHUNK;
+        const int nblk = red_blocks(n3, true);
         const size_t vec64 = (size_t)S * n3 * sizeof(double2);
         const size_t kvec = (size_t)S * n3 * (fp64 ? sizeof(double2) : sizeof(float2));
         c->e64.ensure(vec64); c->b64.ensure(vec64); c->x64.ensure(vec64); c->r64.ensure(vec64);

@@ -20,6 +20,8 @@
 // per system (independent of how many systems share a launch) writes
 // partial sums; consumers add them in block order.  Partial sums of FP32
 // vectors are accumulated in FP32 inside a block.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "solve.h"
@@ -54,6 +56,43 @@ __device__ __forceinline__ void block_sum(T (&v)[K]) {
     __syncthreads();
 }
 
+// Sums four values over the warp: every lane receives the total of v[lane & 3].
+// Lanes trade the values they drop, so the tree takes 6 additions where four
+// separate trees take 20: an FP64 addition of a warp occupies the pipe for 16
+// cycles.
+template <typename T> __device__ __forceinline__ T warp_sum4(const T (&v)[4]) {
+    const int lane = threadIdx.x & 31;
+    const bool hi = lane & 1, up = lane & 2;
+    T a = hi ? v[1] : v[0], b = hi ? v[3] : v[2];
+    a += __shfl_xor_sync(0xffffffffu, hi ? v[0] : v[1], 1);
+    b += __shfl_xor_sync(0xffffffffu, hi ? v[2] : v[3], 1);
+    T t = up ? b : a;
+    t += __shfl_xor_sync(0xffffffffu, up ? a : b, 2);
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
+}
+
+// Partial sums of a reduction block: the RT = red_threads<T>() adjacent threads
+// that took it, in a block of G such groups; part[0..3] is written by the
+// group's first lanes (with `write`).  Every thread of the block calls it; a
+// following call needs a barrier between (sh is reused).
+template <typename T, int G> __device__ __forceinline__ void group_sum4(const T (&v)[4], double* part, bool write) {
+    constexpr int RT = red_threads<T>(), NW = RT / 32;
+    static_assert(NW <= 8, "one lane per warp and value");
+    __shared__ T sh[G * NW * 4];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, grp = threadIdx.x / RT;
+    const T t = warp_sum4(v);
+    if (lane < 4) sh[wid * 4 + lane] = t;
+    __syncthreads();
+    if (wid % NW == 0) {
+        T w = lane < NW * 4 ? sh[grp * NW * 4 + lane] : (T)0;
+#pragma unroll
+        for (int o = 4; o < NW * 4; o <<= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+        if (write && lane < 4) part[lane] = w;
+    }
+}
+
 // part[s][blk][0..3] = (Re sum a.b, Im sum a.b, sum |a|^2, sum |b|^2)   (a.b unconjugated)
 template <typename Rl>
 __global__ void k_dot(int n3, int nblk, const cx<Rl>* __restrict__ a, const cx<Rl>* __restrict__ b, double* part,
@@ -61,7 +100,7 @@ __global__ void k_dot(int n3, int nblk, const cx<Rl>* __restrict__ a, const cx<R
     const int s = blockIdx.y, blk = blockIdx.x;
     if (active && !active[s]) return;
     const size_t off = (size_t)s * n3;
-    const int i0 = blk * RED_CHUNK, i1 = min(n3, i0 + RED_CHUNK);
+    const int chunk = red_chunk(n3, sizeof(Rl) == 8), i0 = blk * chunk, i1 = min(n3, i0 + chunk);
     Rl v[4] = {0, 0, 0, 0};
     for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
         const cx<Rl> x = a[off + i], y = b[off + i];
@@ -70,26 +109,24 @@ __global__ void k_dot(int n3, int nblk, const cx<Rl>* __restrict__ a, const cx<R
         v[2] += x.x * x.x + x.y * x.y;
         v[3] += y.x * y.x + y.y * y.y;
     }
-    block_sum<Rl, 4>(v);
-    if (threadIdx.x == 0) {
-        double* p = part + ((size_t)s * nblk + blk) * 4;
-        p[0] = v[0]; p[1] = v[1]; p[2] = v[2]; p[3] = v[3];
-    }
+    group_sum4<Rl, 1>(v, part + ((size_t)s * nblk + blk) * 4, true);
 }
 
-// Sums part[s][b][0..3] over the blocks b < nblk: lane l adds blocks l, l+32,
-// ... in order, then a fixed shuffle tree adds the lanes.  Called by all 32
-// lanes of a warp; every lane receives the sums.  The order depends only on
-// nblk, so a system's result does not depend on the other systems.
+// Sums part[s][b][0..3] over the blocks b < nblk: lane l adds value l & 3 of
+// the blocks l / 4, l / 4 + 8, ... in order, then a fixed shuffle tree adds the
+// lanes.  Called by all 32 lanes of a warp; every lane receives the sums.  The
+// order depends only on nblk, so a system's result does not depend on the
+// other systems.
 __device__ __forceinline__ void warp_sum_parts(const double* part, int s, int nblk, double (&o)[4]) {
     const int lane = threadIdx.x & 31;
-    const double2* p = reinterpret_cast<const double2*>(part + (size_t)s * nblk * 4);
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-    for (int b = lane; b < nblk; b += 32) {
-        const double2 u = p[2 * b], v = p[2 * b + 1];
-        a0 += u.x; a1 += u.y; a2 += v.x; a3 += v.y;
-    }
-    o[0] = warp_sum(a0); o[1] = warp_sum(a1); o[2] = warp_sum(a2); o[3] = warp_sum(a3);
+    const double* p = part + (size_t)s * nblk * 4 + lane;
+    double t = 0.0;
+#pragma unroll 4
+    for (int b = lane >> 2; b < nblk; b += 8, p += 32) t += __ldcg(p);
+#pragma unroll
+    for (int d = 4; d < 32; d <<= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) o[q] = __shfl_sync(0xffffffffu, t, q);
 }
 
 // Warp-per-system kernels: 4 systems per 128-thread block.
@@ -167,7 +204,7 @@ __global__ void k_lanczos(KrylovArgs<Rl> k, int n) {
     const cx<Rl>* v = k.V[n & 1];
     const cx<Rl>* vp = k.V[(n + 1) & 1];
     const size_t off = (size_t)s * k.n3;
-    const int i0 = blk * RED_CHUNK, i1 = min(k.n3, i0 + RED_CHUNK);
+    const int chunk = red_chunk(k.n3, sizeof(Rl) == 8), i0 = blk * chunk, i1 = min(k.n3, i0 + chunk);
     Rl acc[4] = {0, 0, 0, 0};
     for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
         const cx<Rl> t = k.W[off + i] - al * v[off + i] - be * vp[off + i];
@@ -176,11 +213,7 @@ __global__ void k_lanczos(KrylovArgs<Rl> k, int n) {
         acc[1] += 2 * t.x * t.y;
         acc[2] += t.x * t.x + t.y * t.y;
     }
-    block_sum<Rl, 4>(acc);
-    if (threadIdx.x == 0) {
-        double* p = k.part_b + ((size_t)s * k.nblk + blk) * 4;
-        p[0] = acc[0]; p[1] = acc[1]; p[2] = acc[2]; p[3] = 0.0;
-    }
+    group_sum4<Rl, 1>(acc, k.part_b + ((size_t)s * k.nblk + blk) * 4, true);
 }
 
 template <typename Rl>
@@ -293,7 +326,7 @@ static inline dim3 vec_grid(int n3, int S) {
 template <typename Rl>
 void launch_qmr_init(const KrylovArgs<Rl>& k, cudaStream_t st) {
     count_launch();
-    k_dot<Rl><<<dim3(k.nblk, k.S), RED_THREADS, 0, st>>>(k.n3, k.nblk, k.V[1], k.V[1], k.part_a, k.active);
+    k_dot<Rl><<<dim3(k.nblk, k.S), red_threads<Rl>(), 0, st>>>(k.n3, k.nblk, k.V[1], k.V[1], k.part_a, k.active);
     count_launch();
     k_qmr_start<Rl><<<warp_blocks(k.S), 128, 0, st>>>(k);
     count_launch();
@@ -304,10 +337,10 @@ template <typename Rl>
 void launch_qmr_post_matvec(const KrylovArgs<Rl>& k, int n, bool dot_done, cudaStream_t st) {
     if (!dot_done) {
         count_launch();
-        k_dot<Rl><<<dim3(k.nblk, k.S), RED_THREADS, 0, st>>>(k.n3, k.nblk, k.V[n & 1], k.W, k.part_a, k.active);
+        k_dot<Rl><<<dim3(k.nblk, k.S), red_threads<Rl>(), 0, st>>>(k.n3, k.nblk, k.V[n & 1], k.W, k.part_a, k.active);
     }
     count_launch();
-    k_lanczos<Rl><<<dim3(k.nblk, k.S), RED_THREADS, 0, st>>>(k, n);
+    k_lanczos<Rl><<<dim3(k.nblk, k.S), red_threads<Rl>(), 0, st>>>(k, n);
     count_launch();
     k_qmr_step<Rl><<<warp_blocks(k.S), 128, 0, st>>>(k);
     count_launch();
@@ -345,19 +378,17 @@ __global__ void k_qmr2_start(KrylovArgs<Rl> k) {
     if (threadIdx.x & 31) return;
     Qmr2State q;
     const double rho = sqrt(o[2]);
-    q.bnorm = rho;
     q.rho = rho;
-    q.tau = rho;
-    q.gam = 1.0;
-    q.th = 0.0;
+    q.th2 = 0.0;
+    q.ig2 = 1.0;
     q.cd = 0.0;
     q.eta = make_double2(-1, 0);
     q.cp = make_double2(0, 0);
     q.iters = 0;
     q.qres = 1.0;
     q.status = 0;
-    q.delta = make_double2(1, 0);
     q.inv_rho = 0.0;
+    q.delta = make_double2(1, 0);
     if (rho > 0.0) {
         q.inv_rho = 1.0 / rho;
         // v_1^T v_1 ~ 0 is caught by the first step, after k_qmr2_scale has
@@ -367,6 +398,8 @@ __global__ void k_qmr2_start(KrylovArgs<Rl> k) {
         q.status = 1;
         q.qres = 0.0;
     }
+    q.nd2 = abs2_(q.delta);
+    q.idel = (1.0 / q.nd2) * conj_(q.delta);
     if (q.status != 0) {
         k.active[s] = 0;
         atomicSub(k.n_active, 1);
@@ -391,6 +424,36 @@ __global__ void k_qmr2_scale(KrylovArgs<Rl> k) {
     }
 }
 
+// Entries of a vector pass that a thread loads before it stores any (the
+// vectors may alias for all the compiler knows, so it keeps their order).
+template <typename Rl> constexpr int vec_batch() { return sizeof(Rl) == 4 ? 4 : 2; }
+
+// v~ = W - beta v (into W) on the entries i, i + st, ... < i1, with the sums of
+// v~.v~ and |v~|^2.
+template <typename Rl>
+__device__ __forceinline__ void qmr2_lanczos_at(const KrylovArgs<Rl>& k, cx<Rl> be, size_t off, int i, int i1, int st,
+                                                Rl (&acc)[4]) {
+    constexpr int B = vec_batch<Rl>();
+    using C = cx<Rl>;
+    C* W = k.W + off;
+    const C* V = k.V[1] + off;
+    for (; i < i1; i += B * st) {
+        C w[B], v[B];
+#pragma unroll
+        for (int u = 0; u < B; ++u)
+            if (i + u * st < i1) { w[u] = W[i + u * st]; v[u] = V[i + u * st]; }
+#pragma unroll
+        for (int u = 0; u < B; ++u) {
+            if (i + u * st >= i1) break;
+            const C t = w[u] - be * v[u];
+            W[i + u * st] = t;
+            acc[0] += t.x * t.x - t.y * t.y;
+            acc[1] += 2 * t.x * t.y;
+            acc[2] += t.x * t.x + t.y * t.y;
+        }
+    }
+}
+
 // v~ = A p_n - beta_n v_n (into W), beta_n = eps_n / delta_n with eps_n from
 // part_a; partial sums of v~.v~ and |v~|^2 into part_b
 template <typename Rl>
@@ -401,25 +464,112 @@ __global__ void k_qmr2_lanczos(KrylovArgs<Rl> k) {
     if (threadIdx.x < 32) {
         double o[4];
         warp_sum_parts(k.part_a, s, k.nblk_a, o);
-        if (threadIdx.x == 0) sc = cdiv(make_double2(o[0], o[1]), k.qmr2[s].delta);
+        if (threadIdx.x == 0) sc = make_double2(o[0], o[1]) * k.qmr2[s].idel;
     }
     __syncthreads();
     const cx<Rl> be = cvt<cx<Rl>>(sc);
-    const cx<Rl>* v = k.V[1];
     const size_t off = (size_t)s * k.n3;
-    const int i0 = blk * RED_CHUNK, i1 = min(k.n3, i0 + RED_CHUNK);
+    const int chunk = red_chunk(k.n3, sizeof(Rl) == 8), i0 = blk * chunk, i1 = min(k.n3, i0 + chunk);
     Rl acc[4] = {0, 0, 0, 0};
-    for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-        const cx<Rl> t = k.W[off + i] - be * v[off + i];
-        k.W[off + i] = t;
-        acc[0] += t.x * t.x - t.y * t.y;
-        acc[1] += 2 * t.x * t.y;
-        acc[2] += t.x * t.x + t.y * t.y;
+    qmr2_lanczos_at<Rl>(k, be, off, i0 + threadIdx.x, i1, blockDim.x, acc);
+    group_sum4<Rl, 1>(acc, k.part_b + ((size_t)s * k.nblk + blk) * 4, true);
+}
+
+// Coefficients of the vector update of one system.
+struct Qmr2Coef {
+    double2 eta, cp;
+    double cd, ir;
+};
+
+// The scalars of iteration n, in three parts by one warp (every lane the same
+// inputs).  A warp's FP64 instruction takes its scheduler's share of the pipe
+// for 64 cycles whether one lane works or 32, so a division or a root costs
+// half a microsecond and the chain between the sums of v~ and the update is what
+// the kernel waits for: Qmr2Pre holds what eps_n = p_n^T A p_n alone decides,
+// qmr2_coefs takes one reciprocal root for both of its arguments and shares the
+// products among the lanes, and qmr2_finish, what only the next iteration and
+// the stopping test need, runs beside the update.
+// (16 divisions, 3 roots and 2 hypots in a row before: 15 us an iteration.)
+struct Qmr2Pre {
+    double2 ieps;         // 1 / eps_n
+    double2 E;            // eta_n / gamma_n^2 = -(rho_n / gamma_{n-1}^2) eta_{n-1} / beta_n
+    double kth;           // theta_n^2 / rho_{n+1}^2
+    bool ok;              // beta_n != 0 and finite
+};
+__device__ __forceinline__ bool finite_(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ Qmr2Pre qmr2_pre(const Qmr2State& q, double2 eps) {
+    Qmr2Pre p;
+    const double r = 1.0 / abs2_(eps);
+    p.ieps = r * conj_(eps);
+    p.E = -(q.rho * q.ig2) * (q.eta * (q.delta * p.ieps));
+    p.kth = q.nd2 * r * q.ig2;
+    p.ok = finite_(r) && p.kth > 0.0;
+    return p;
+}
+// ob = (Re, Im of v~^T v~, |v~|^2).  Returns whether the update applies.
+__device__ __forceinline__ bool qmr2_coefs(const Qmr2State& q, const Qmr2Pre& p, const double (&ob)[4], Qmr2Coef& c) {
+    const int lane = threadIdx.x & 31;
+    const double th2 = ob[2] * p.kth;
+    const double y = rsqrt(lane == 0 ? ob[2] : 1.0 + th2);
+    const double y0 = __shfl_sync(0xffffffffu, y, 0), g = __shfl_sync(0xffffffffu, y, 1);
+    const double ir = ob[2] > 0.0 ? y0 : 0.0, g2 = g * g;
+    // lanes 0..5: eta.x, eta.y, cd = g^2 (E.x, E.y, theta^2); cp.x, cp.y, ir = ir ((v~^T v~) / eps, 1)
+    const double a = lane == 0 ? p.E.x : lane == 1 ? p.E.y : lane == 2 ? q.th2 : lane == 5 ? 1.0 : ob[0];
+    const double b = lane == 3 ? p.ieps.x : lane == 4 ? p.ieps.y : 1.0;
+    const double d = lane == 3 ? -p.ieps.y : lane == 4 ? p.ieps.x : 0.0;
+    double t = a * b;
+    if (lane == 3 || lane == 4) t += ob[1] * d;
+    t *= lane < 3 ? g2 : ir;
+    c.eta = make_double2(__shfl_sync(0xffffffffu, t, 0), __shfl_sync(0xffffffffu, t, 1));
+    c.cd = __shfl_sync(0xffffffffu, t, 2);
+    c.cp = make_double2(__shfl_sync(0xffffffffu, t, 3), __shfl_sync(0xffffffffu, t, 4));
+    c.ir = __shfl_sync(0xffffffffu, t, 5);
+    return p.ok && finite_(ob[2]) && finite_(th2) && finite_(c.eta.x) && finite_(c.eta.y);
+}
+// The state of iteration n + 1; returns whether the system goes on.
+__device__ __forceinline__ bool qmr2_finish(Qmr2State& q, const Qmr2Pre& p, const double (&ob)[4], const Qmr2Coef& c,
+                                            bool upd, double tol, int max_iter) {
+    q.iters += 1;
+    if (!upd) {
+        // eps_n = 0 (or not finite): the coupled recurrences break down and
+        // this iteration's update is undefined; x keeps its previous value
+        q.status = 3;
+        return false;
     }
-    block_sum<Rl, 4>(acc);
-    if (threadIdx.x == 0) {
-        double* p = k.part_b + ((size_t)s * k.nblk + blk) * 4;
-        p[0] = acc[0]; p[1] = acc[1]; p[2] = acc[2]; p[3] = 0.0;
+    q.eta = c.eta; q.cp = c.cp; q.cd = c.cd; q.inv_rho = c.ir;
+    const double th2 = ob[2] * p.kth;
+    q.qres *= sqrt(th2 / (1.0 + th2));                // theta_n gamma_n
+    q.th2 = th2;
+    q.ig2 = 1.0 + th2;
+    if (!(ob[2] > 0.0)) {           // invariant subspace reached: this update is exact
+        q.status = 1;
+        return false;
+    }
+    q.rho = ob[2] * c.ir;
+    const double ir2 = c.ir * c.ir;
+    q.delta = make_double2(ob[0] * ir2, ob[1] * ir2);
+    q.nd2 = abs2_(q.delta);
+    if (!(q.nd2 >= 1e-60)) { q.status = 3; return false; }
+    q.idel = (1.0 / q.nd2) * conj_(q.delta);
+    if (q.qres <= tol) { q.status = 1; return false; }
+    if (q.iters >= max_iter) { q.status = 2; return false; }
+    return true;
+}
+// delta_1 = v_1^T v_1 / |v_1|^2 below the rounding floor of the vector
+// precision: the Lanczos process breaks down at its start (beta_1 would be
+// eps_1 / rounding noise, and tau collapse to a false convergence with
+// x ~ 0).  Stop with status 3 and the zero x that k_qmr2_scale wrote.
+template <typename Rl> __device__ __forceinline__ bool qmr2_breaks_at_start(const Qmr2State& q) {
+    const double floor2 = sizeof(Rl) == 4 ? 1e-10 : 1e-24;
+    return q.iters == 0 && !(q.nd2 >= floor2);
+}
+template <typename Rl> __device__ __forceinline__ void qmr2_store(const KrylovArgs<Rl>& k, int s, const Qmr2State& q,
+                                                                  bool upd, bool next) {
+    k.qmr2[s] = q;
+    k.upd[s] = upd;
+    if (!next) {
+        k.active[s] = 0;
+        atomicSub(k.n_active, 1);
     }
 }
 
@@ -435,97 +585,158 @@ __global__ void k_qmr2_step(KrylovArgs<Rl> k) {
     double oa[4], ob[4];
     warp_sum_parts(k.part_a, s, k.nblk_a, oa);
     warp_sum_parts(k.part_b, s, k.nblk, ob);
-    if (!lead) return;
     Qmr2State q = k.qmr2[s];
-    // delta_1 = v_1^T v_1 / |v_1|^2 below the rounding floor of the vector
-    // precision: the Lanczos process breaks down at its start (beta_1 would be
-    // eps_1 / rounding noise, and tau collapse to a false convergence with
-    // x ~ 0).  Stop with status 3 and the zero x that k_qmr2_scale wrote.
-    const double delta_floor = sizeof(Rl) == 4 ? 1e-5 : 1e-12;
-    if (q.iters == 0 && !(cabs_(q.delta) >= delta_floor)) {
-        q.iters = 1;
-        q.status = 3;
-        k.qmr2[s] = q;
-        k.upd[s] = 0;
-        k.active[s] = 0;
-        atomicSub(k.n_active, 1);
-        return;
-    }
-    const double2 eps = make_double2(oa[0], oa[1]);
-    const double2 beta = cdiv(eps, q.delta);
-    const double abeta = cabs_(beta);
-    const double rho_n = sqrt(ob[2]);
-    q.iters += 1;
-    int next = 1, upd = 1;
-    if (!(abeta > 0.0) || !(rho_n == rho_n)) {
-        // eps_n = 0 (or not finite): the coupled recurrences break down and
-        // this iteration's update is undefined; x keeps its previous value
-        q.status = 3; next = 0; upd = 0;
-    } else {
-        const double th = rho_n / (q.gam * abeta);
-        const double g = 1.0 / sqrt(1.0 + th * th);
-        const double f = q.rho * g * g / (q.gam * q.gam);
-        q.eta = -(f * cdiv(q.eta, beta));
-        q.cd = (q.th * g) * (q.th * g);
-        q.tau = q.tau * th * g;
-        q.qres = q.tau / q.bnorm;
-        q.th = th;
-        q.gam = g;
-        if (rho_n > 0.0) {
-            const double2 dn = make_double2(ob[0] / (rho_n * rho_n), ob[1] / (rho_n * rho_n));
-            q.cp = cdiv(rho_n * dn, eps);
-            q.inv_rho = 1.0 / rho_n;
-            q.rho = rho_n;
-            if (!(cabs_(dn) >= 1e-30)) { q.status = 3; next = 0; }
-            q.delta = dn;
-        } else {                    // invariant subspace reached: the update below is exact
-            q.cp = make_double2(0, 0);
-            q.inv_rho = 0.0;
-            q.status = 1; next = 0;
-        }
-        if (next && q.qres <= (k.eps_sys ? k.eps_sys[s] : k.eps)) { q.status = 1; next = 0; }
-        if (next && q.iters >= k.max_iter) { q.status = 2; next = 0; }
-        if (!(q.qres == q.qres) || !(q.eta.x == q.eta.x) || !(q.eta.y == q.eta.y)) {   // NaN guard
-            q.status = 3; next = 0; upd = 0;
-        }
-    }
-    k.qmr2[s] = q;
-    k.upd[s] = upd;
-    if (!next) {
-        k.active[s] = 0;
-        atomicSub(k.n_active, 1);
-    }
+    const Qmr2Pre pre = qmr2_pre(q, make_double2(oa[0], oa[1]));
+    Qmr2Coef c;
+    const bool upd = qmr2_coefs(q, pre, ob, c) && !qmr2_breaks_at_start<Rl>(q);
+    const bool next = qmr2_finish(q, pre, ob, c, upd, k.eps_sys ? k.eps_sys[s] : k.eps, k.max_iter);
+    __syncwarp();
+    if (lead) qmr2_store<Rl>(k, s, q, upd, next);
 }
 
+// The update's coefficients in the vectors' precision.
+template <typename Rl> struct Qmr2Vec {
+    cx<Rl> eta, cp;
+    Rl cd, ir;
+    __device__ Qmr2Vec(double2 e, double2 p, double c, double i) : eta(cvt<cx<Rl>>(e)), cp(cvt<cx<Rl>>(p)), cd((Rl)c), ir((Rl)i) {}
+};
 // d_n = eta_n p_n + cd d_{n-1}; x += d_n; v_{n+1} = v~ / rho_{n+1};
 // p_{n+1} = v_{n+1} - cp p_n
+template <typename Rl>
+__device__ __forceinline__ void qmr2_update_at(const KrylovArgs<Rl>& k, const Qmr2Vec<Rl>& q, size_t off, int i, int i1,
+                                               int st) {
+    constexpr int B = vec_batch<Rl>();
+    using C = cx<Rl>;
+    C *P = k.P[0] + off, *D = k.P[1] + off, *X = k.X + off, *V = k.V[1] + off;
+    const C* W = k.W + off;
+    for (; i < i1; i += B * st) {
+        C p[B], d[B], x[B], w[B];
+#pragma unroll
+        for (int u = 0; u < B; ++u) {
+            const int j = i + u * st;
+            if (j < i1) { p[u] = P[j]; d[u] = D[j]; x[u] = X[j]; w[u] = W[j]; }
+        }
+#pragma unroll
+        for (int u = 0; u < B; ++u) {
+            const int j = i + u * st;
+            if (j >= i1) break;
+            const C dn = q.eta * p[u] + q.cd * d[u];
+            D[j] = dn;
+            X[j] = x[u] + dn;
+            const C vn = q.ir * w[u];
+            V[j] = vn;
+            P[j] = vn - q.cp * p[u];
+        }
+    }
+}
 template <typename Rl>
 __global__ void k_qmr2_update(KrylovArgs<Rl> k) {
     const int s = blockIdx.y;
     if (!k.upd[s]) return;
+    const Qmr2State& st = k.qmr2[s];
+    const Qmr2Vec<Rl> q(st.eta, st.cp, st.cd, st.inv_rho);
+    qmr2_update_at<Rl>(k, q, (size_t)s * k.n3, blockIdx.x * blockDim.x + threadIdx.x, k.n3, gridDim.x * blockDim.x);
+}
+
+// The three kernels above as one, a cluster of blocks per system: the blocks
+// take the same reduction blocks, G at a time, and meet once, at the cluster
+// barrier, for the sums of v~.  A warp of its own in every block works out the
+// scalars.  Same sums in the same order, so a system's bits do not depend on
+// which form ran.
+//
+// What bounds it: FP64, the pipe (28 instructions an entry); FP32, the L2; for
+// small vectors the launch, the barrier and the scalars' chain.  At most 56
+// registers, so that two clusters share their SMs: 24 systems at one block per
+// SM ran in two rounds (with loads one by one, 1548 us in place of 1285 for 12
+// iterations of 32^3 cells).  Three kernels before: 44 us an iteration of one
+// FP64 system of 2775 entries (now about 10), 28 us of 24 FP32 systems of 51768.
+template <typename Rl, int G>
+__global__ void __launch_bounds__(G * red_threads<Rl>() + 32, G * red_threads<Rl>() == 512 ? 2 : 4) k_qmr2_post(KrylovArgs<Rl> k) {
     using C = cx<Rl>;
-    const Qmr2State& q = k.qmr2[s];
-    const C eta = cvt<C>(q.eta), cp = cvt<C>(q.cp);
-    const Rl cd = (Rl)q.cd, ir = (Rl)q.inv_rho;
+    constexpr int RT = red_threads<Rl>();
+    namespace cg = cooperative_groups;
+    const cg::cluster_group cl = cg::this_cluster();
+    const int s = blockIdx.y, grp = threadIdx.x / RT, lane = threadIdx.x & 31;
+    const bool scalars = threadIdx.x >= G * RT;
+    if (!k.active[s]) return;                         // the whole cluster: active changes after its barrier
+    __shared__ double2 be_s;
+    __shared__ Qmr2Coef co;
+    __shared__ int upd_s;
     const size_t off = (size_t)s * k.n3;
-    C* v = k.V[1];
-    C* p = k.P[0];
-    C* d = k.P[1];
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < k.n3; i += gridDim.x * blockDim.x) {
-        const C pn = p[off + i];
-        const C dn = eta * pn + cd * d[off + i];
-        d[off + i] = dn;
-        k.X[off + i] = k.X[off + i] + dn;
-        const C vn = ir * k.W[off + i];
-        v[off + i] = vn;
-        p[off + i] = vn - cp * pn;
+    const int chunk = red_chunk(k.n3, sizeof(Rl) == 8), step = gridDim.x * G, b0 = blockIdx.x * G + grp;
+    if (scalars) {
+        double oa[4], ob[4];
+        warp_sum_parts(k.part_a, s, k.nblk_a, oa);
+        Qmr2State q = k.qmr2[s];
+        const double2 eps = make_double2(oa[0], oa[1]);
+        if (lane == 0) be_s = eps * q.idel;
+        __syncthreads();
+        const Qmr2Pre pre = qmr2_pre(q, eps);
+        for (int base = 0; base < k.nblk; base += step) {
+            if (base) __syncthreads();
+            __syncthreads();                          // in group_sum4
+        }
+        cl.sync();
+        warp_sum_parts(k.part_b, s, k.nblk, ob);
+        Qmr2Coef c;
+        const bool upd = qmr2_coefs(q, pre, ob, c) && !qmr2_breaks_at_start<Rl>(q);
+        if (lane == 0) { co = c; upd_s = upd; }
+        __syncthreads();
+        if (blockIdx.x == 0) {
+            const bool next = qmr2_finish(q, pre, ob, c, upd, k.eps_sys ? k.eps_sys[s] : k.eps, k.max_iter);
+            if (lane == 0) qmr2_store<Rl>(k, s, q, upd, next);
+        }
+        return;
     }
+    __syncthreads();
+    const C be = cvt<C>(be_s);
+    for (int base = 0; base < k.nblk; base += step) {
+        const int blk = base + b0, i0 = blk * chunk, i1 = min(k.n3, i0 + chunk);
+        Rl acc[4] = {0, 0, 0, 0};
+        qmr2_lanczos_at<Rl>(k, be, off, i0 + threadIdx.x % RT, i1, RT, acc);
+        if (base) __syncthreads();
+        group_sum4<Rl, G>(acc, k.part_b + ((size_t)s * k.nblk + blk) * 4, blk < k.nblk);
+    }
+    cl.sync();
+    __syncthreads();
+    if (!upd_s) return;
+    const Qmr2Vec<Rl> c(co.eta, co.cp, co.cd, co.ir);
+    for (int blk = b0; blk < k.nblk; blk += step) {
+        const int i0 = blk * chunk, i1 = min(k.n3, i0 + chunk);
+        qmr2_update_at<Rl>(k, c, off, i0 + threadIdx.x % RT, i1, RT);
+    }
+}
+
+// One kernel where a cluster of eight SMs does the vectors of a system about as
+// fast as the whole chip would: up to 65536 entries in FP32 (4.6 us of L2
+// traffic per SM); in FP64, whose pipe needs 0.9 ns an entry of a cluster, up to
+// 8192 entries, or 32768 when there are systems enough to fill the SMs.  Inner
+// solves, three kernels and one: 24 FP32 systems of 32^3 cells 1469 and 1285 us;
+// whole requests of 16 such systems 77.9 and 65.6 ms, of one FP64 system of 12^3
+// cells 71.6 and 49.8 ms.
+template <typename Rl> static bool qmr2_one_kernel(const KrylovArgs<Rl>& k) {
+    if (sizeof(Rl) == 4) return k.n3 <= 65536;
+    return k.n3 <= 8192 || (k.n3 <= 32768 && k.S >= 16);
+}
+
+template <typename Rl, int G> static void qmr2_post_launch(const KrylovArgs<Rl>& k, int cl, cudaStream_t st) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(cl, k.S);
+    cfg.blockDim = dim3(G * red_threads<Rl>() + 32);
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = cl;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_qmr2_post<Rl, G>, k);
 }
 
 template <typename Rl>
 void launch_qmr2_init(const KrylovArgs<Rl>& k, cudaStream_t st) {
     count_launch();
-    k_dot<Rl><<<dim3(k.nblk, k.S), RED_THREADS, 0, st>>>(k.n3, k.nblk, k.V[1], k.V[1], k.part_a, k.active);
+    k_dot<Rl><<<dim3(k.nblk, k.S), red_threads<Rl>(), 0, st>>>(k.n3, k.nblk, k.V[1], k.V[1], k.part_a, k.active);
     count_launch();
     k_qmr2_start<Rl><<<warp_blocks(k.S), 128, 0, st>>>(k);
     count_launch();
@@ -536,10 +747,20 @@ template <typename Rl>
 void launch_qmr2_post_matvec(const KrylovArgs<Rl>& k, bool dot_done, cudaStream_t st) {
     if (!dot_done) {
         count_launch();
-        k_dot<Rl><<<dim3(k.nblk, k.S), RED_THREADS, 0, st>>>(k.n3, k.nblk, k.P[0], k.W, k.part_a, k.active);
+        k_dot<Rl><<<dim3(k.nblk, k.S), red_threads<Rl>(), 0, st>>>(k.n3, k.nblk, k.P[0], k.W, k.part_a, k.active);
+    }
+    if (qmr2_one_kernel<Rl>(k)) {
+        int cl = 1;
+        while (cl < 8 && cl < k.nblk) cl *= 2;
+        const int g = (k.nblk + cl - 1) / cl;
+        count_launch();
+        if (g > 2 && sizeof(Rl) == 8) qmr2_post_launch<Rl, sizeof(Rl) == 8 ? 4 : 2>(k, cl, st);
+        else if (g > 1) qmr2_post_launch<Rl, 2>(k, cl, st);
+        else qmr2_post_launch<Rl, 1>(k, cl, st);
+        return;
     }
     count_launch();
-    k_qmr2_lanczos<Rl><<<dim3(k.nblk, k.S), RED_THREADS, 0, st>>>(k);
+    k_qmr2_lanczos<Rl><<<dim3(k.nblk, k.S), red_threads<Rl>(), 0, st>>>(k);
     count_launch();
     k_qmr2_step<Rl><<<warp_blocks(k.S), 128, 0, st>>>(k);
     count_launch();
@@ -580,7 +801,7 @@ __global__ void k_dotc(int n3, int nblk, const cx<Rl>* __restrict__ a, const cx<
     const int s = blockIdx.y, blk = blockIdx.x;
     if (active && !active[s]) return;
     const size_t off = (size_t)s * n3;
-    const int i0 = blk * RED_CHUNK, i1 = min(n3, i0 + RED_CHUNK);
+    const int chunk = red_chunk(n3, sizeof(Rl) == 8), i0 = blk * chunk, i1 = min(n3, i0 + chunk);
     Rl v[4] = {0, 0, 0, 0};
     for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
         const cx<Rl> x = a[off + i], y = b[off + i];
@@ -588,11 +809,7 @@ __global__ void k_dotc(int n3, int nblk, const cx<Rl>* __restrict__ a, const cx<
         v[1] += x.x * y.y - x.y * y.x;
         v[2] += x.x * x.x + x.y * x.y;
     }
-    block_sum<Rl, 4>(v);
-    if (threadIdx.x == 0) {
-        double* p = part + ((size_t)s * nblk + blk) * 4;
-        p[0] = v[0]; p[1] = v[1]; p[2] = v[2]; p[3] = 0.0;
-    }
+    group_sum4<Rl, 1>(v, part + ((size_t)s * nblk + blk) * 4, true);
 }
 
 // r^ = r, p = r, x = 0
@@ -673,7 +890,7 @@ __global__ void k_bicg_x(KrylovArgs<Rl> k) {
     __syncthreads();
     const cx<Rl> al = cvt<cx<Rl>>(sc[0]), om = cvt<cx<Rl>>(sc[1]);
     const size_t off = (size_t)s * k.n3;
-    const int i0 = blk * RED_CHUNK, i1 = min(k.n3, i0 + RED_CHUNK);
+    const int chunk = red_chunk(k.n3, sizeof(Rl) == 8), i0 = blk * chunk, i1 = min(k.n3, i0 + chunk);
     Rl acc[4] = {0, 0, 0, 0};
     for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
         const cx<Rl> sv = k.R[off + i];
@@ -685,11 +902,7 @@ __global__ void k_bicg_x(KrylovArgs<Rl> k) {
         acc[1] += h.x * r.y - h.y * r.x;
         acc[2] += r.x * r.x + r.y * r.y;
     }
-    block_sum<Rl, 4>(acc);
-    if (threadIdx.x == 0) {
-        double* p = k.part_a + ((size_t)s * k.nblk + blk) * 4;
-        p[0] = acc[0]; p[1] = acc[1]; p[2] = acc[2]; p[3] = 0.0;
-    }
+    group_sum4<Rl, 1>(acc, k.part_a + ((size_t)s * k.nblk + blk) * 4, true);
 }
 
 template <typename Rl>
@@ -741,7 +954,7 @@ void launch_bicg_init(const KrylovArgs<Rl>& k, cudaStream_t st) {
     count_launch();
     k_bicg_copy<Rl><<<vec_grid(k.n3, k.S), 256, 0, st>>>(k);
     count_launch();
-    k_dotc<Rl><<<dim3(k.nblk, k.S), RED_THREADS, 0, st>>>(k.n3, k.nblk, k.R, k.R, k.part_a, k.active);
+    k_dotc<Rl><<<dim3(k.nblk, k.S), red_threads<Rl>(), 0, st>>>(k.n3, k.nblk, k.R, k.R, k.part_a, k.active);
     count_launch();
     k_bicg_start<Rl><<<warp_blocks(k.S), 128, 0, st>>>(k);
 }
@@ -749,7 +962,7 @@ void launch_bicg_init(const KrylovArgs<Rl>& k, cudaStream_t st) {
 template <typename Rl>
 void launch_bicg_stage1(const KrylovArgs<Rl>& k, cudaStream_t st) {
     count_launch();
-    k_dotc<Rl><<<dim3(k.nblk, k.S), RED_THREADS, 0, st>>>(k.n3, k.nblk, k.Rh, k.Vb, k.part_a, k.active);
+    k_dotc<Rl><<<dim3(k.nblk, k.S), red_threads<Rl>(), 0, st>>>(k.n3, k.nblk, k.Rh, k.Vb, k.part_a, k.active);
     count_launch();
     k_bicg_s<Rl><<<vec_grid(k.n3, k.S), 256, 0, st>>>(k);
 }
@@ -757,9 +970,9 @@ void launch_bicg_stage1(const KrylovArgs<Rl>& k, cudaStream_t st) {
 template <typename Rl>
 void launch_bicg_stage2(const KrylovArgs<Rl>& k, cudaStream_t st) {
     count_launch();
-    k_dotc<Rl><<<dim3(k.nblk, k.S), RED_THREADS, 0, st>>>(k.n3, k.nblk, k.Tb, k.R, k.part_b, k.active);
+    k_dotc<Rl><<<dim3(k.nblk, k.S), red_threads<Rl>(), 0, st>>>(k.n3, k.nblk, k.Tb, k.R, k.part_b, k.active);
     count_launch();
-    k_bicg_x<Rl><<<dim3(k.nblk, k.S), RED_THREADS, 0, st>>>(k);
+    k_bicg_x<Rl><<<dim3(k.nblk, k.S), red_threads<Rl>(), 0, st>>>(k);
     count_launch();
     k_bicg_step<Rl><<<warp_blocks(k.S), 128, 0, st>>>(k);
     count_launch();
@@ -790,17 +1003,13 @@ __global__ void k_rhs_init(LatticeDev L, int S, const double2* e, const double2*
 __global__ void k_norms2(int n3, int nblk, const double2* a, const double2* b, double* part) {
     const int s = blockIdx.y, blk = blockIdx.x;
     const size_t off = (size_t)s * n3;
-    const int i0 = blk * RED_CHUNK, i1 = min(n3, i0 + RED_CHUNK);
-    double v[2] = {0, 0};
+    const int chunk = red_chunk(n3, true), i0 = blk * chunk, i1 = min(n3, i0 + chunk);
+    double v[4] = {0, 0, 0, 0};
     for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
         v[0] += abs2_(a[off + i]);
         v[1] += abs2_(b[off + i]);
     }
-    block_sum<double, 2>(v);
-    if (threadIdx.x == 0) {
-        double* p = part + ((size_t)s * nblk + blk) * 4;
-        p[0] = v[0]; p[1] = v[1]; p[2] = 0; p[3] = 0;
-    }
+    group_sum4<double, 1>(v, part + ((size_t)s * nblk + blk) * 4, true);
 }
 
 __global__ void k_residual_check(int S, int nblk, const double* part, double eps, double eps_floor, double safety,
@@ -862,7 +1071,7 @@ void launch_rhs_init(const LatticeDev& L, int S, const double2* e, const double2
 }
 void launch_norms2(int S, int n3, int nblk, const double2* a, const double2* b, double* part, cudaStream_t st) {
     count_launch();
-    k_norms2<<<dim3(nblk, S), RED_THREADS, 0, st>>>(n3, nblk, a, b, part);
+    k_norms2<<<dim3(nblk, S), red_threads<double>(), 0, st>>>(n3, nblk, a, b, part);
 }
 void launch_residual_check(int S, int nblk, const double* part, double eps, double eps_floor, double safety,
                            double* res, double* rnorm, int* outer, int* n_outer, double* eps_sys, cudaStream_t st) {

@@ -21,17 +21,18 @@ struct QmrState {
     int status;           // 0 running, 1 converged, 2 iteration limit, 3 breakdown
 };
 
-// Per-system scalars of QMR from coupled two-term recurrences (FP64).
+// Per-system scalars of QMR from coupled two-term recurrences (FP64), kept in
+// the form that leaves the fewest divisions and roots between two kernels.
 struct Qmr2State {
     double2 delta;        // delta_n = v_n^T v_n (unconjugated)
+    double2 idel;         // 1 / delta_n
     double2 eta;          // d_n = eta_n p_n + cd d_{n-1}
     double2 cp;           // p_{n+1} = v_{n+1} - cp p_n
+    double nd2;           // |delta_n|^2
     double rho;           // rho_n = ||v~_n||
-    double gam, th;       // gamma_{n-1}, theta_{n-1}
+    double th2, ig2;      // theta_{n-1}^2, 1 / gamma_{n-1}^2 = 1 + theta_{n-1}^2
     double cd;            // (theta_{n-1} gamma_n)^2
-    double tau;           // quasi-residual norm tau_n
     double inv_rho;       // 1 / rho_{n+1}: v_{n+1} = v~_{n+1} / rho_{n+1}
-    double bnorm;         // ||b||
     double qres;          // tau_n / ||b||
     int iters;
     int status;           // 0 running, 1 converged, 2 iteration limit, 3 breakdown
@@ -48,7 +49,7 @@ struct BicgState {
 template <typename Rl>
 struct KrylovArgs {
     int S, n3, nblk;               // systems, vector length 3N, reduction blocks per system
-    int nblk_a;                    // partial sums of v^T (A v) per system in part_a (3 Nx when the matvec writes them)
+    int nblk_a;                    // partial sums of v^T (A v) per system in part_a (matvec_dot_parts when the matvec writes them)
     cx<Rl>* V[2];                  // Lanczos vectors (slot n % 2 holds v_n)
     cx<Rl>* P[3];                  // QMR directions (slot n % 3 holds p_n)
     cx<Rl>* W;                     // A v_n, then v~_{n+1}
@@ -68,8 +69,17 @@ struct KrylovArgs {
     int max_iter;
 };
 
-constexpr int RED_THREADS = 256;
-constexpr int RED_CHUNK = 4096;    // vector entries per reduction block
+// Reduction blocks: how many vector entries each sums, with how many threads.
+// They depend on the vector alone, so a system's sums do not depend on the
+// batch.  FP64 vectors take small blocks: an SM issues one FP64 warp
+// instruction every 16 cycles, so 4096 entries on one SM take 20 us where the
+// whole chip needs a few hundred ns; long ones take fewer (every block of the
+// next kernel adds all partial sums).
+__host__ __device__ constexpr int red_chunk(int n3, bool fp64) {
+    return !fp64 || n3 > 131072 ? 4096 : n3 > 32768 ? 1024 : 256;
+}
+template <typename Rl> __host__ __device__ constexpr int red_threads() { return sizeof(Rl) == 8 ? 128 : 256; }
+inline int red_blocks(int n3, bool fp64) { return (n3 + red_chunk(n3, fp64) - 1) / red_chunk(n3, fp64); }
 
 // QMR (complex symmetric, Freund 1992): start from the rhs stored in V[1].
 template <typename Rl> void launch_qmr_init(const KrylovArgs<Rl>& k, cudaStream_t st);
