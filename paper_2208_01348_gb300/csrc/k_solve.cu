@@ -641,8 +641,7 @@ __global__ void k_qmr2_update(KrylovArgs<Rl> k) {
 // The three kernels above as one, a cluster of blocks per system: the blocks
 // take the same reduction blocks, G at a time, and meet once, at the cluster
 // barrier, for the sums of v~.  A warp of its own in every block works out the
-// scalars.  Same sums in the same order, so a system's bits do not depend on
-// which form ran.
+// scalars.
 //
 // What bounds it: FP64, the pipe (28 instructions an entry); FP32, the L2; for
 // small vectors the launch, the barrier and the scalars' chain.  At most 56
@@ -709,14 +708,14 @@ __global__ void __launch_bounds__(G * red_threads<Rl>() + 32, G * red_threads<Rl
 
 // One kernel where a cluster of eight SMs does the vectors of a system about as
 // fast as the whole chip would: up to 65536 entries in FP32 (4.6 us of L2
-// traffic per SM); in FP64, whose pipe needs 0.9 ns an entry of a cluster, up to
-// 8192 entries, or 32768 when there are systems enough to fill the SMs.  Inner
+// traffic per SM) and 32768 in FP64 (0.44 ns of its pipe an entry, against the
+// 12 us or so of three kernels).  By the vector alone: the two forms do not round
+// alike everywhere, and a system's bits do not depend on the batch.  Inner
 // solves, three kernels and one: 24 FP32 systems of 32^3 cells 1469 and 1285 us;
 // whole requests of 16 such systems 77.9 and 65.6 ms, of one FP64 system of 12^3
 // cells 71.6 and 49.8 ms.
 template <typename Rl> static bool qmr2_one_kernel(const KrylovArgs<Rl>& k) {
-    if (sizeof(Rl) == 4) return k.n3 <= 65536;
-    return k.n3 <= 8192 || (k.n3 <= 32768 && k.S >= 16);
+    return k.n3 <= (sizeof(Rl) == 4 ? 65536 : 32768);
 }
 
 template <typename Rl, int G> static void qmr2_post_launch(const KrylovArgs<Rl>& k, int cl, cudaStream_t st) {

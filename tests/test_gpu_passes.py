@@ -130,3 +130,35 @@ def test_lanczos_sums_of_split_slabs(dd, ctx, dims, prec):
     dd.eels_matvec_dev(ctx, p, x.data_ptr(), r.data_ptr(), 1, st)
     # the quasi-residual underestimates the residual by at most sqrt(iterations + 1) <= 71
     assert float(torch.linalg.vector_norm(r - b) / torch.linalg.vector_norm(b)) < 71 * eps
+
+
+@pytest.mark.parametrize("dims,prec", [((11, 11, 31), "FP64"), ((11, 11, 31), "MIXED"), ((3, 4, 5), "FP64"),
+                                       ((24, 20, 30), "FP64"), ((30, 27, 28), "MIXED")])
+def test_qmr2_bits_do_not_depend_on_the_batch(dd, ctx, dims, prec):
+    """3N entries decide how an iteration's vectors are cut up and whether one kernel
+    or three run them: 16 systems together and the first and last of them alone
+    give the same bits."""
+    import torch
+    occ, d_nm, eps_h = _occ(dims, 1, True), 1.5, 1.0 + 0j
+    dd.eels_set_grid(ctx, occ, d_nm)
+    n, S = int(np.count_nonzero(occ)), 16
+    e = np.linspace(3.3, 4.0, S)
+    eps_p = np.stack([[I.drude(v)] for v in e])
+    p = getattr(dd, "EELS_" + prec)
+    dt, eps = (torch.complex128, 1e-9) if prec == "FP64" else (torch.complex64, 1e-5)
+    g = torch.Generator(device="cuda").manual_seed(6)
+    b = torch.randn((S, 3, n), generator=g, device="cuda", dtype=dt)
+    st = torch.cuda.current_stream().cuda_stream
+
+    def solve(i0, i1):
+        dd.eels_prepare_operator(ctx, e[i0:i1], eps_p[i0:i1], np.full(i1 - i0, eps_h))
+        x = torch.zeros_like(b[i0:i1])
+        status, iters = dd.eels_krylov_solve_dev(ctx, p, dd.EELS_QMR2, b[i0:i1].data_ptr(), x.data_ptr(), i1 - i0, eps,
+                                                 2000, st)
+        torch.cuda.synchronize()
+        assert (status == 1).all()
+        return x, iters
+    x, iters = solve(0, S)
+    for i in (0, S - 1):
+        xi, it = solve(i, i + 1)
+        assert it[0] == iters[i] and torch.equal(xi[0], x[i])
