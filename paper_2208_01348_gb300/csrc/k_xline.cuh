@@ -29,8 +29,22 @@ template <typename Rl> __device__ __forceinline__ const cx<Rl>* xline_tw(const L
 template <> __device__ __forceinline__ const double2* xline_tw<double>(const LatticeDev& L) { return L.tw64x; }
 template <> __device__ __forceinline__ const float2* xline_tw<float>(const LatticeDev& L) { return L.tw32x; }
 
-template <typename Rl, int RE, int RO>
-__global__ void __launch_bounds__(256, sizeof(Rl) == 4 && RO <= 10 ? (RO <= 6 ? 3 : 2) : 1)
+template <typename C> __device__ __forceinline__ C shfl_c(C v, int l) {
+    v.x = __shfl_sync(0xffffffffu, v.x, l);
+    v.y = __shfl_sync(0xffffffffu, v.y, l);
+    return v;
+}
+
+// SPLIT (FP64, lattices of at most 65536 padded points): the middle step of a
+// line and butterfly is shared by three lanes, one a component.  Such a grid gives
+// a scheduler one or two warps, and a warp's FP64 instruction takes 32 cycles of
+// it (64 where it waits for the one before), so the step's 312 instructions in a
+// row are the kernel: 12^3 cells, one system, 47 -> 39 us a matvec; 16 systems of 11 x 11 x
+// 31 the same either way.  Where there are warps enough it costs more than it
+// gives: 8 systems of 32^3 cells 957 -> 1040 us a matvec, and in FP32 (shuffles on
+// top of the shared-memory accesses) 4 of 79^3 468 -> 660 us.
+template <typename Rl, int RE, int RO, bool SPLIT>
+__global__ void __launch_bounds__(SPLIT ? 512 : 256, sizeof(Rl) == 4 && RO <= 10 ? (RO <= 6 ? 3 : 2) : 1)
 k_xline(LatticeDev L, MatvecArgs<Rl> a, int lgw) {
     using C = cx<Rl>;
     constexpr int LEN = RE * RO, HX = LEN / 2 + 1;
@@ -48,6 +62,8 @@ k_xline(LatticeDev L, MatvecArgs<Rl> a, int lgw) {
     const int nw = min(W, Mz - kz0), hz = Mz / 2;
     const bool ny = ky > L.My / 2;
     const size_t cs = (size_t)L.Hy * L.Hx * L.Hz;
+    const int lane = threadIdx.x & 31, gl = lane / 3, c = lane - 3 * gl;
+    const int l1 = min(31, 3 * gl + (c + 1) % 3), l2 = min(31, 3 * gl + (c + 2) % 3);
     int cur = -1;
     for (int s = s0; s < s1; ++s) {
         if (a.active && !a.active[s]) continue;
@@ -70,18 +86,42 @@ k_xline(LatticeDev L, MatvecArgs<Rl> a, int lgw) {
             __pipeline_wait_prior(0);
         }
         __syncthreads();
-        xline_mid<RE, RO>(A, lgw, nw, tw, threadIdx.x, blockDim.x, [&](int w, int kx, C (&g)[6]) {
-            const int kz = kz0 + w, kxr = kx > LEN / 2 ? LEN - kx : kx;
-            const bool nx = kx > LEN / 2, nz = kz > hz;
-            const C* d = STAGE ? D + (kxr << lgw) + w : Ds + (size_t)kxr * L.Hz + (nz ? Mz - kz : kz);
-            const size_t st = STAGE ? (size_t)(HX << lgw) : cs;
-            g[0] = d[0];
-            g[1] = flip_c(d[st], nx != ny);
-            g[2] = flip_c(d[2 * st], nx != nz);
-            g[3] = d[3 * st];
-            g[4] = flip_c(d[4 * st], ny != nz);
-            g[5] = d[5 * st];
-        });
+        if constexpr (SPLIT) {
+            // ten triples of lanes a warp, one triple a line and butterfly
+            for (int g0 = (threadIdx.x >> 5) * 10; g0 < RE << lgw; g0 += (blockDim.x >> 5) * 10) {
+                const int g = g0 + gl, w = g & (W - 1), j = g >> lgw, kz = kz0 + w;
+                const bool ok = lane < 30 && j < RE && w < nw, nz = kz > hz;
+                C v[RO];
+                C* d = A + (ok ? j * 3 * W + c * W + w : 0);
+                const C* tj = tw + (ok ? j : 0);
+                xline_mid_in<RE, RO>(d, 3 * W, tj, v);
+#pragma unroll
+                for (int r = 0; r < RO; ++r) {
+                    const int kx = j + r * RE, kxr = kx > LEN / 2 ? LEN - kx : kx;
+                    const bool nx = kx > LEN / 2;
+                    const C next = shfl_c(v[r], l1), prev = shfl_c(v[r], l2);
+                    if (!ok) continue;
+                    const C* q = Ds + (size_t)kxr * L.Hz + (nz ? Mz - kz : kz);
+                    v[r] = q[sym_own(c) * cs] * v[r] +
+                           flip_c(q[sym_next(c) * cs], sym_flip(sym_next(c), nx, ny, nz)) * next +
+                           flip_c(q[sym_prev(c) * cs], sym_flip(sym_prev(c), nx, ny, nz)) * prev;
+                }
+                if (ok) xline_mid_out<RE, RO>(d, 3 * W, tj, v);
+            }
+        } else {
+            xline_mid<RE, RO>(A, lgw, nw, tw, threadIdx.x, blockDim.x, [&](int w, int kx, C (&g)[6]) {
+                const int kz = kz0 + w, kxr = kx > LEN / 2 ? LEN - kx : kx;
+                const bool nx = kx > LEN / 2, nz = kz > hz;
+                const C* d = STAGE ? D + (kxr << lgw) + w : Ds + (size_t)kxr * L.Hz + (nz ? Mz - kz : kz);
+                const size_t st = STAGE ? (size_t)(HX << lgw) : cs;
+                g[0] = d[0];
+                g[1] = flip_c(d[st], nx != ny);
+                g[2] = flip_c(d[2 * st], nx != nz);
+                g[3] = d[3 * st];
+                g[4] = flip_c(d[4 * st], ny != nz);
+                g[5] = d[5 * st];
+            });
+        }
         __syncthreads();
         xline_2<RE, RO>(A, lgw, Nx, threadIdx.x, blockDim.x, [&](int c, int w, int ix, C v) {
             if (w < nw) U0[c * cstride + (size_t)ix * Mz + w] = v;
@@ -93,6 +133,10 @@ template <typename Rl> static size_t xline_smem(const LatticeDev& L, int w) {
     return (size_t)(L.Mx + 3 * w * L.Mx + (sizeof(Rl) == 4 ? 6 * w * (L.Mx / 2 + 1) : 0)) * sizeof(cx<Rl>);
 }
 template <typename Rl> bool xline_fits(const LatticeDev& L, int w) { return xline_smem<Rl>(L, w) <= 224 * 1024; }
+
+template <typename Rl> static bool xline_split(const LatticeDev& L) {
+    return sizeof(Rl) == 8 && (long long)L.Mx * L.My * L.Mz <= 65536;
+}
 
 template <typename Rl> void launch_xline(const LatticeDev& L, const MatvecArgs<Rl>& a, int w, cudaStream_t st) {
     int lgw = 0;
@@ -106,22 +150,30 @@ template <typename Rl> void launch_xline(const LatticeDev& L, const MatvecArgs<R
     b.spb = std::max(1, std::min(a.spb, a.S));
     while (b.spb > 1 && (long long)tiles * ((a.S + b.spb - 1) / b.spb) < 1216) b.spb /= 2;
     const dim3 grid((L.Mz + (1 << lgw) - 1) >> lgw, L.My, (a.S + b.spb - 1) / b.spb);
-    const int nthr = std::min(256, std::max(64, ((L.qx.Re << lgw) + 31) / 32 * 32));
+    const bool split = xline_split<Rl>(L);
+    const int items = L.qx.Re << lgw;
+    const int nthr = split ? std::min(512, std::max(64, (items + 9) / 10 * 32))
+                           : std::min(256, std::max(64, (items + 31) / 32 * 32));
     const size_t sm = xline_smem<Rl>(L, 1 << lgw);
     count_launch();
     switch (L.Mx) {
-#define XL(RE, RO) case RE * RO: k_xline<Rl, RE, RO><<<grid, nthr, sm, st>>>(L, b, lgw); break;
+#define XL(RE, RO)                                                                            \
+    case RE * RO:                                                                             \
+        if (split) k_xline<Rl, RE, RO, sizeof(Rl) == 8><<<grid, nthr, sm, st>>>(L, b, lgw);  \
+        else k_xline<Rl, RE, RO, false><<<grid, nthr, sm, st>>>(L, b, lgw);                  \
+        break;
         EELS_PLANS(XL)
 #undef XL
         default: break;
     }
 }
 
+template <typename K> static void prepare_xline(K k) {
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);
+    cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+}
 template <typename Rl> void prepare_xline_kernels() {
-#define XL(RE, RO)                                                                                         \
-    cudaFuncSetAttribute(k_xline<Rl, RE, RO>, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);  \
-    cudaFuncSetAttribute(k_xline<Rl, RE, RO>, cudaFuncAttributePreferredSharedMemoryCarveout,            \
-                         (int)cudaSharedmemCarveoutMaxShared);
+#define XL(RE, RO) prepare_xline(k_xline<Rl, RE, RO, false>); prepare_xline(k_xline<Rl, RE, RO, sizeof(Rl) == 8>);
     EELS_PLANS(XL)
 #undef XL
 }

@@ -79,6 +79,32 @@ HD void xline_mid(C* A, int lgw, int nw, const C* tw, int tid, int nthr, Dh dhat
         }
     }
 }
+// The middle step of one component of one line, as three lanes share it: up to
+// the end of the forward transform, and from the start of the inverse one.  d is
+// row j of the component and line, es the row length, tw the twiddle (0, j).
+template <int RE, int RO, typename C> HD void xline_mid_in(const C* d, int es, const C* tw, C (&v)[RO]) {
+#pragma unroll
+    for (int r = 0; r < RO; ++r) {
+        v[r] = d[(size_t)r * RE * es];
+        if (r) v[r] = v[r] * tw[r * RE];
+    }
+    Dft<RO, false, C>::run(v);
+}
+template <int RE, int RO, typename C> HD void xline_mid_out(C* d, int es, const C* tw, C (&v)[RO]) {
+    Dft<RO, true, C>::run(v);
+#pragma unroll
+    for (int r = 0; r < RO; ++r) {
+        if (r) v[r] = v[r] * conj_(tw[r * RE]);
+        d[(size_t)r * RE * es] = v[r];
+    }
+}
+// Row c of the symmetric tensor xx xy xz yy yz zz, in the order of the
+// components c, c + 1, c + 2 (mod 3), and the sign of an off-diagonal entry
+// where the frequency lies in the upper half along (x, y, z).
+HD int sym_own(int c) { return c == 0 ? 0 : c == 1 ? 3 : 5; }
+HD int sym_next(int c) { return c == 0 ? 1 : c == 1 ? 4 : 2; }
+HD int sym_prev(int c) { return c == 0 ? 2 : c == 1 ? 1 : 4; }
+HD bool sym_flip(int i, bool nx, bool ny, bool nz) { return i == 1 ? nx != ny : i == 2 ? nx != nz : ny != nz; }
 // Step 2 inverse: out(c, w, ix, value) for ix < n.
 template <int RE, int RO, typename C, class Out>
 HD void xline_2(const C* A, int lgw, int n, int tid, int nthr, Out out) {

@@ -140,7 +140,7 @@ template <typename Rl> static void slab_rows(int L, int n, int g) {
 }
 
 // The x pass: transform, symmetric product per frequency, transform back.
-template <typename Rl, int RE, int RO> static void x_lines(int n, int nw, int nthr) {
+template <typename Rl, int RE, int RO> static void x_lines(int n, int nw, int nthr, bool split) {
     using C = cx<Rl>;
     constexpr int L = RE * RO, lgw = 2, W = 1 << lgw;
     const std::vector<C> tw = twiddles<C>(make_plan2(L));
@@ -152,10 +152,26 @@ template <typename Rl, int RE, int RO> static void x_lines(int n, int nw, int nt
         xline_1<RE, RO>(A.data(), lgw, n, t, nthr, [&](int c, int w, int i) {
             return w < nw ? x[at(c, w, i)] : mk<C>(0.0, 0.0);
         });
-    for (int t = 0; t < nthr; ++t)
-        xline_mid<RE, RO>(A.data(), lgw, nw, tw.data(), t, nthr, [&](int w, int k, C (&g)[6]) {
-            for (int c = 0; c < 6; ++c) g[c] = D[((size_t)c * L + k) * W + w];
-        });
+    if (split) {
+        for (int w = 0; w < nw; ++w)
+            for (int j = 0; j < RE; ++j) {
+                C v[3][RO], u[3][RO];
+                auto row = [&](int c) { return A.data() + j * 3 * W + c * W + w; };
+                for (int c = 0; c < 3; ++c) xline_mid_in<RE, RO>(row(c), 3 * W, tw.data() + j, v[c]);
+                for (int c = 0; c < 3; ++c)
+                    for (int r = 0; r < RO; ++r) {
+                        auto g = [&](int i) { return D[((size_t)i * L + j + r * RE) * W + w]; };
+                        u[c][r] = g(sym_own(c)) * v[c][r] + g(sym_next(c)) * v[(c + 1) % 3][r] +
+                                  g(sym_prev(c)) * v[(c + 2) % 3][r];
+                    }
+                for (int c = 0; c < 3; ++c) xline_mid_out<RE, RO>(row(c), 3 * W, tw.data() + j, u[c]);
+            }
+    } else {
+        for (int t = 0; t < nthr; ++t)
+            xline_mid<RE, RO>(A.data(), lgw, nw, tw.data(), t, nthr, [&](int w, int k, C (&g)[6]) {
+                for (int c = 0; c < 6; ++c) g[c] = D[((size_t)c * L + k) * W + w];
+            });
+    }
     for (int t = 0; t < nthr; ++t)
         xline_2<RE, RO>(A.data(), lgw, n, t, nthr, [&](int c, int w, int i, C v) { if (w < nw) y[at(c, w, i)] = v; });
     const int sym[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
@@ -215,7 +231,7 @@ template <int RE, int RO> static void one_length() {
         if (n < 1 || 2 * n - 1 > L) continue;
         slab_columns<float>(L, n, 5, 64); slab_columns<double>(L, n, 1, 96);
         slab_rows<float>(L, n, 3); slab_rows<double>(L, n, 1);
-        x_lines<float, RE, RO>(n, 4, 64); x_lines<double, RE, RO>(n, 3, 96);
+        x_lines<float, RE, RO>(n, 4, 64, false); x_lines<double, RE, RO>(n, 3, 96, false); x_lines<double, RE, RO>(n, 3, 64, true);
         if (2 * n <= L) { dhat_line<RE, RO>(n, false, 64); dhat_line<RE, RO>(n, true, 64); }
     }
 }
