@@ -293,6 +293,8 @@ template <bool INV, typename C> struct Dft<12, INV, C> : DftPfa<3, 4, INV, C> {}
 template <bool INV, typename C> struct Dft<14, INV, C> : DftPfa<2, 7, INV, C> {};
 template <bool INV, typename C> struct Dft<15, INV, C> : DftPfa<3, 5, INV, C> {};
 template <bool INV, typename C> struct Dft<16, INV, C> : DftCt<4, 4, INV, C> {};
+template <bool INV, typename C> struct Dft<18, INV, C> : DftPfa<2, 9, INV, C> {};
+template <bool INV, typename C> struct Dft<20, INV, C> : DftPfa<4, 5, INV, C> {};
 template <> HD double sin_2pi<25>(int k) {
     const double c[13] = {0, 0.248689887164854788243, 0.481753674101715274987, 0.684547105928688673732,
                           0.844327925502015078549, K_S5_1, 0.998026728428271561952, 0.982287250728688681085,

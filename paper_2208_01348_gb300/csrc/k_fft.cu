@@ -391,6 +391,7 @@ void launch_matvec(const LatticeDev& L, const MatvecArgs<Rl>& a, cudaStream_t st
     slab_launch_any<Rl>(L, a, true, st);
 }
 
+void prepare_dhat_kernels();
 void prepare_far_kernels();
 void prepare_xreg_kernels();
 
@@ -411,6 +412,7 @@ void prepare_kernels() {
     allow_smem(k_slab_inv_r<16, true, false>);
     allow_smem(k_slab_inv_r<16, false, true>);
     allow_smem(k_slab_inv_r<16, false, false>);
+    prepare_dhat_kernels();
     prepare_far_kernels();
     prepare_slab_kernels<float>();
     prepare_slab_kernels<double>();

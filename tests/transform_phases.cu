@@ -199,17 +199,21 @@ template <typename Rl, int RE, int RO> static void x_lines(int n, int nw, int nt
 // One axis of the D-hat build: an even or odd sequence from its octant.
 template <int RE, int RO> static void dhat_line(int n, bool odd, int nthr) {
     constexpr int L = RE * RO, W = 3, ES = 4;
-    const std::vector<double2> tw = twiddles<double2>(make_plan2(L));
-    std::vector<double2> A((size_t)L * ES);
+    const std::vector<double2> tw = twiddles<double2>(make_plan2(L));   // the rows j <= RO/2 are read
+    constexpr int rows = DhatLine<RE, RO>::ROWS;
+    std::vector<double2> A((size_t)rows * ES), F_((size_t)(L / 2 + 1) * W);
+    std::vector<int> seen(F_.size(), 0);
     std::vector<std::vector<Z>> g(W, std::vector<Z>(n));
     for (auto& l : g) for (Z& v : l) v = rnd();
     if (odd) for (auto& l : g) l[0] = 0;
-    auto in = [&](int w, int i) { return to_c<double2>(g[w][i] * (i ? 1.0L : 0.5L)); };
-    for (int t = 0; t < nthr; ++t) {
-        if (odd) dhat_1<RE, RO, true>(A.data(), ES, W, n, t, nthr, in);
-        else dhat_1<RE, RO, false>(A.data(), ES, W, n, t, nthr, in);
-    }
-    for (int t = 0; t < nthr; ++t) dhat_2<RE, RO>(A.data(), ES, W, tw.data(), t, nthr);
+    for (int t = 0; t < nthr; ++t)
+        dhat_1<RE, RO>(A.data(), ES, W, n, odd, t, nthr, [&](int w, int i) { return to_c<double2>(g[w][i]); });
+    for (int t = 0; t < nthr; ++t)
+        dhat_2<RE, RO>(A.data(), ES, W, odd, tw.data(), t, nthr, [&](int w, int k, double2 v) {
+            F_[(size_t)k * W + w] = v;
+            ++seen[(size_t)k * W + w];
+        });
+    for (int v : seen) if (v != 1) { printf("D-hat: L=%d: an output %d times\n", L, v); ++g_bad; break; }
     Err e;
     for (int w = 0; w < W; ++w) {
         std::vector<Z> full(L);
@@ -218,9 +222,9 @@ template <int RE, int RO> static void dhat_line(int n, bool odd, int nthr) {
             if (i) full[L - i] += odd ? -g[w][i] : g[w][i];
         }
         const std::vector<Z> F = dft(full, L, false);
-        for (int k = 0; k <= L / 2; ++k) e.add(to_z(dhat_fold(A.data(), ES, L, k, w, odd)), F[k]);
+        for (int k = 0; k <= L / 2; ++k) e.add(to_z(F_[(size_t)k * W + w]), F[k]);
     }
-    // the odd part of a two-entry line is all rounding when it vanishes: skip empty references
+    // an odd line of one entry vanishes
     if (e.n > 0) e.check(odd ? "D-hat odd" : "D-hat even", L, n, 1.12e-16, 2);
 }
 
