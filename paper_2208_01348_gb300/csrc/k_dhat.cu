@@ -10,7 +10,7 @@
 // (dhat.cuh) to the frequencies 0 <= k <= M/2 that are kept: 3 N^2 lines per
 // component in place of 12 N^2, half of each line's butterflies, and N^3
 // exponentials in place of 8 N^3.  The FP64 pipe bounds it (the arrays of one
-// energy of 64^3 cells are 25 MB): 0.32 ms per energy of 64^3 cells, against 0.46
+// energy of 64^3 cells are 25 MB): 0.33 ms per energy of 64^3 cells, against 0.46
 // ms with half-filled lines transformed whole and 2.2 ms for the padded
 // lattice.  The last axis writes D-hat in the layouts that the x passes read.
 #include <algorithm>

@@ -133,6 +133,11 @@ __device__ __forceinline__ void warp_sum_parts(const double* part, int s, int nb
 __device__ __forceinline__ int warp_system() { return blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); }
 static inline unsigned warp_blocks(int S) { return (unsigned)((S + 3) / 4); }
 
+// 1 / a for the scalars of the Lanczos processes, whose vectors have unit norm
+// (no intermediate over- or underflow): one division, where a quotient by
+// Smith's algorithm takes three in a row.
+__device__ __forceinline__ double2 crecip(double2 a) { return (1.0 / abs2_(a)) * conj_(a); }
+
 // ------------------------------------------------------------------- QMR
 template <typename Rl>
 __global__ void k_qmr_start(KrylovArgs<Rl> k) {
@@ -195,7 +200,7 @@ __global__ void k_lanczos(KrylovArgs<Rl> k, int n) {
         warp_sum_parts(k.part_a, s, k.nblk_a, o);
         if (threadIdx.x == 0) {
             const QmrState& q = k.qmr[s];
-            sc[0] = cdiv(make_double2(o[0], o[1]), q.delta);
+            sc[0] = make_double2(o[0], o[1]) * crecip(q.delta);
             sc[1] = q.beta;
         }
     }
@@ -244,26 +249,27 @@ __global__ void k_qmr_step(KrylovArgs<Rl> k) {
         atomicSub(k.n_active, 1);
         return;
     }
-    const double2 alpha = cdiv(make_double2(oa[0], oa[1]), q.delta);
-    const double rho_n = sqrt(ob[2]);
+    const double2 idel = crecip(q.delta);
+    const double2 alpha = make_double2(oa[0], oa[1]) * idel;
+    const double ir = ob[2] > 0.0 ? rsqrt(ob[2]) : ob[2], rho_n = ob[2] * ir;   // NaN stays NaN
     // Givens: apply rotations n-2, n-1 to the column (beta_n, alpha_n, rho_{n+1})
     const double2 theta = q.s2 * q.beta;
     const double2 tmp = q.c2 * q.beta;
     const double2 eta = q.c1 * tmp + q.s1 * alpha;
     const double2 mu = q.c1 * alpha - conj_(q.s1) * tmp;
-    const double amu = cabs_(mu);
+    const double amu2 = abs2_(mu);
     double c;
-    double2 sn, r;
-    if (amu == 0.0) {
-        c = 0.0; sn = make_double2(1, 0); r = make_double2(rho_n, 0);
+    double2 sn, rinv;
+    if (amu2 == 0.0) {
+        c = 0.0; sn = make_double2(1, 0); rinv = make_double2(1.0 / rho_n, 0);
     } else {
-        const double ra = hypot(amu, rho_n);
-        const double2 ph = (1.0 / amu) * mu;
-        c = amu / ra; sn = (rho_n / ra) * ph; r = ra * ph;
+        const double ia = rsqrt(amu2), ira = rsqrt(amu2 + ob[2]);
+        const double2 ph = ia * mu;
+        c = amu2 * ia * ira; sn = (rho_n * ira) * ph; rinv = ira * conj_(ph);
     }
     q.theta = theta;
     q.eta = eta;
-    q.rinv = cdiv(make_double2(1, 0), r);
+    q.rinv = rinv;
     q.t = c * q.tau;
     q.tau = -(conj_(sn) * q.tau);
     q.c2 = q.c1; q.s2 = q.s1; q.c1 = c; q.s1 = sn;
@@ -271,10 +277,10 @@ __global__ void k_qmr_step(KrylovArgs<Rl> k) {
     q.qres = cabs_(q.tau) / q.bnorm;
     int next = 1;
     if (rho_n > 0.0) {
-        const double2 dn = make_double2(ob[0] / (rho_n * rho_n), ob[1] / (rho_n * rho_n));
-        q.beta = cdiv(rho_n * dn, q.delta);
-        q.inv_rho = 1.0 / rho_n;
-        if (cabs_(dn) < 1e-30) { q.status = 3; next = 0; }
+        const double2 dn = (ir * ir) * make_double2(ob[0], ob[1]);
+        q.beta = (rho_n * dn) * idel;
+        q.inv_rho = ir;
+        if (abs2_(dn) < 1e-60) { q.status = 3; next = 0; }
         q.delta = dn;
     } else {
         q.inv_rho = 0.0;           // invariant subspace reached: the update below is exact
