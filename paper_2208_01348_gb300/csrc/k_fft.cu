@@ -26,8 +26,6 @@
 
 namespace eels {
 
-constexpr int FFT_THREADS = 256;
-
 template <typename Rl> __device__ __forceinline__ const cx<Rl>* tw_of(const LatticeDev& L, int axis);
 template <> __device__ __forceinline__ const double2* tw_of<double>(const LatticeDev& L, int axis) {
     return axis == 0 ? L.tw64x : (axis == 1 ? L.tw64y : L.tw64z);
@@ -52,17 +50,22 @@ template <> __device__ __forceinline__ const float2* tw_of<float>(const LatticeD
 // every column's occupied cells are contiguous in z, so a dipole's index is
 // the column's base plus iz (no cell-map load).
 // ---------------------------------------------------------------------------
+// 64 points: blocks of 4 warps, seven on an SM, so that the block barriers of
+// one slab are filled by more others (four blocks of 8 warps: 773 -> 733 us a
+// matvec of 200 systems of 32^3 cells, although 28 warps are resident in place
+// of 32); the larger slab of 128 points leaves room for two blocks of 8 warps.
 template <int R> struct SlabR {
     static constexpr int L = 8 * R;
     static constexpr int SLS = R == 8 ? 36 : 68;           // slab row stride
     static constexpr int TILE = R == 8 ? R64_TILE : R128_TILE;
+    static constexpr int THREADS = R == 8 ? 128 : 256, BLOCKS = R == 8 ? 7 : 2;     // per SM
 };
 
 template <int R> struct SlabRSmem {
     float2 tw2[(R - 1) * 8];                     // exp(-2 pi i p k / L) at [k - 1][p]: conflict-free per k
     float2 cf[EELS_MAX_MAT], dg[EELS_MAX_MAT];   // this system's per-material coefficients
     float2 S[SlabR<R>::L * SlabR<R>::SLS];
-    alignas(16) float2 tile[FFT_THREADS / 32][SlabR<R>::TILE];
+    alignas(16) float2 tile[SlabR<R>::THREADS / 32][SlabR<R>::TILE];
     int4 ci[SlabR<R>::L / 2];                    // this slab's column table (contiguous columns)
 };
 
@@ -73,7 +76,7 @@ template <int R> struct SlabRSmem {
 // the z transforms of the current one, so the gather's latency is hidden
 // behind arithmetic instead of opening every item.
 template <int R, bool HALF, bool FAST>
-__global__ void __launch_bounds__(FFT_THREADS, R == 8 ? 4 : 2) k_slab_fwd_r(LatticeDev L, MatvecArgs<float> a) {
+__global__ void __launch_bounds__(SlabR<R>::THREADS, SlabR<R>::BLOCKS) k_slab_fwd_r(LatticeDev L, MatvecArgs<float> a) {
     using C = float2;
     using P = SlabR<R>;
     constexpr int LEN = P::L, SLS = P::SLS;
@@ -181,13 +184,13 @@ __global__ void __launch_bounds__(FFT_THREADS, R == 8 ? 4 : 2) k_slab_fwd_r(Latt
 }
 
 template <int R, bool HALF, bool FAST>
-__global__ void __launch_bounds__(FFT_THREADS, R == 8 ? 4 : 2) k_slab_inv_r(LatticeDev L, MatvecArgs<float> a, float invM) {
+__global__ void __launch_bounds__(SlabR<R>::THREADS, SlabR<R>::BLOCKS) k_slab_inv_r(LatticeDev L, MatvecArgs<float> a, float invM) {
     using C = float2;
     using P = SlabR<R>;
     constexpr int LEN = P::L, SLS = P::SLS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SlabRSmem<R>& sm = *reinterpret_cast<SlabRSmem<R>*>(smem_raw);
-    __shared__ float red[2 * FFT_THREADS / 32];
+    __shared__ float red[2 * SlabR<R>::THREADS / 32];
     const int ix = blockIdx.x, b = blockIdx.y, s = b / 3, c = b % 3;
     if (a.active && !a.active[s]) return;
     const int Ny = L.Ny, Nz = L.Nz, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = lane & 3, p = lane >> 2;
@@ -308,12 +311,12 @@ static void slab_r_launch(const LatticeDev& L, const MatvecArgs<float>& a, bool 
     const size_t sm = sizeof(SlabRSmem<R>);
     const float invM = (float)(1.0 / ((double)L.Mx * L.My * L.Mz));
     if (!inv) {
-        // persistent: the blocks resident at once (2 or 4 per multiprocessor)
+        // persistent: the blocks resident at once
         const int items = a.S * 3 * L.Nx;
-        const int blocks = std::min(items, sm_count() * (R == 8 ? 4 : 2));
-        k_slab_fwd_r<R, HALF, FAST><<<blocks, FFT_THREADS, sm, st>>>(L, a);
+        const int blocks = std::min(items, sm_count() * SlabR<R>::BLOCKS);
+        k_slab_fwd_r<R, HALF, FAST><<<blocks, SlabR<R>::THREADS, sm, st>>>(L, a);
     } else {
-        k_slab_inv_r<R, HALF, FAST><<<dim3(L.Nx, a.S * 3), FFT_THREADS, sm, st>>>(L, a, invM);
+        k_slab_inv_r<R, HALF, FAST><<<dim3(L.Nx, a.S * 3), SlabR<R>::THREADS, sm, st>>>(L, a, invM);
     }
 }
 
