@@ -95,5 +95,14 @@ __host__ __device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
 }
 __host__ __device__ __forceinline__ double cabs_(double2 a) { return hypot(a.x, a.y); }
 
+#ifdef __CUDACC__
+// Programmatic dependent launch (launch_dep): a kernel may start while the one
+// before it drains, and waits, before it touches memory, until it has finished;
+// then it lets the next one start.
+__device__ __forceinline__ void dep_wait(int on) {
+    if (on) asm volatile("griddepcontrol.wait;\n griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
+
 // Fixed-size per-system scalars of the solve (device resident).
 #define EELS_MAX_MAT 8

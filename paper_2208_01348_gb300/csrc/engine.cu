@@ -613,6 +613,7 @@ KrylovArgs<Rl> krylov_args(eels_ctx* c, int S, const eels_opts* o, double eps) {
     k.eps = eps;
     k.eps_sys = c->eps_sys.as<double>();
     k.max_iter = inner_cap(o, sizeof(Rl) == 4);
+    k.dep = matvec_dep(c->L, S, sizeof(Rl) == 8);
     return k;
 }
 

@@ -290,8 +290,7 @@ template <typename K> static void allow_smem(K kernel) {
 }
 
 // Register-resident slab kernels: FP32 with 64- or 128-point y and z transforms.
-// Multiprocessors of the current device (queried once per device).
-static int sm_count() {
+int sm_count() {
     static int cache[64] = {0};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { cudaGetLastError(); return 132; }
@@ -389,9 +388,11 @@ template <typename Rl> static void xpass_any(const LatticeDev& L, const MatvecAr
 template <typename Rl>
 void launch_matvec(const LatticeDev& L, const MatvecArgs<Rl>& a, cudaStream_t st) {
     // slab (gather, y, z) -> x * D-hat * x -> slab (z, y, scatter)
-    slab_launch_any<Rl>(L, a, false, st);
-    xpass_any<Rl>(L, a, st);
-    slab_launch_any<Rl>(L, a, true, st);
+    MatvecArgs<Rl> b = a;
+    b.dep = matvec_dep(L, a.S, sizeof(Rl) == 8);
+    slab_launch_any<Rl>(L, b, false, st);
+    xpass_any<Rl>(L, b, st);
+    slab_launch_any<Rl>(L, b, true, st);
 }
 
 void prepare_dhat_kernels();
@@ -428,6 +429,11 @@ template void launch_matvec<float>(const LatticeDev&, const MatvecArgs<float>&, 
 template void launch_matvec<double>(const LatticeDev&, const MatvecArgs<double>&, cudaStream_t);
 
 static bool slab_reg(const LatticeDev& L) { return (L.My == 64 && L.Mz == 64) || (L.My == 128 && L.Mz == 128); }
+bool matvec_dep(const LatticeDev& L, int S, bool fp64) {
+    if (!fp64 && (slab_reg(L) || xpass_reg_supported(L))) return false;
+    const long long slabs = 3LL * L.Nx * S * (fp64 ? L.s64.CL : L.s32.CL), lines = (L.Mz + 3) / 4 * (long long)L.My * S;
+    return std::max(slabs, lines) <= sm_count();
+}
 int matvec_dot_parts(const LatticeDev& L, bool fp64) {
     return 3 * L.Nx * (fp64 ? L.s64.CL : slab_reg(L) ? 1 : L.s32.CL);
 }

@@ -72,6 +72,7 @@ __device__ __forceinline__ void slab_tables(const LatticeDev& L, const MatvecArg
 template <typename Rl, bool CLUSTER>
 __global__ void __launch_bounds__(sizeof(Rl) == 4 ? 768 : 512, 1) k_slab_fwd(LatticeDev L, MatvecArgs<Rl> a) {
     using C = cx<Rl>;
+    dep_wait(a.dep);
     const SlabPlan& sp = plan_of<Rl>(L);
     const int CL = CLUSTER ? sp.CL : 1, rank = CLUSTER ? blockIdx.x % CL : 0, ix = CLUSTER ? blockIdx.x / CL : blockIdx.x;
     const int b = blockIdx.y, s = b / 3, c = b % 3;
@@ -162,6 +163,7 @@ __global__ void __launch_bounds__(sizeof(Rl) == 4 ? 768 : 512, 1) k_slab_fwd(Lat
 template <typename Rl, bool CLUSTER>
 __global__ void __launch_bounds__(sizeof(Rl) == 4 ? 768 : 512, 1) k_slab_inv(LatticeDev L, MatvecArgs<Rl> a, Rl invM) {
     using C = cx<Rl>;
+    dep_wait(a.dep);
     const SlabPlan& sp = plan_of<Rl>(L);
     const int CL = CLUSTER ? sp.CL : 1, rank = CLUSTER ? blockIdx.x % CL : 0, ix = CLUSTER ? blockIdx.x / CL : blockIdx.x;
     const int b = blockIdx.y, s = b / 3, c = b % 3;
@@ -278,23 +280,13 @@ void launch_slab(const LatticeDev& L, const MatvecArgs<Rl>& a, bool inv, cudaStr
     count_launch();
     if (p.CL == 1) {
         const dim3 grid(L.Nx, a.S * 3);
-        if (!inv) k_slab_fwd<Rl, false><<<grid, p.nthr, sm, st>>>(L, a);
-        else k_slab_inv<Rl, false><<<grid, p.nthr, sm, st>>>(L, a, invM);
+        if (!inv) launch_dep(a.dep, k_slab_fwd<Rl, false>, grid, p.nthr, sm, 1, st, L, a);
+        else launch_dep(a.dep, k_slab_inv<Rl, false>, grid, p.nthr, sm, 1, st, L, a, invM);
         return;
     }
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(L.Nx * p.CL, a.S * 3);
-    cfg.blockDim = dim3(p.nthr);
-    cfg.dynamicSmemBytes = sm;
-    cfg.stream = st;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = p.CL;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    if (!inv) cudaLaunchKernelEx(&cfg, k_slab_fwd<Rl, true>, L, a);
-    else cudaLaunchKernelEx(&cfg, k_slab_inv<Rl, true>, L, a, invM);
+    const dim3 grid(L.Nx * p.CL, a.S * 3);
+    if (!inv) launch_dep(a.dep, k_slab_fwd<Rl, true>, grid, p.nthr, sm, p.CL, st, L, a);
+    else launch_dep(a.dep, k_slab_inv<Rl, true>, grid, p.nthr, sm, p.CL, st, L, a, invM);
 }
 template <typename K> static void allow(K k) {
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);

@@ -658,6 +658,7 @@ __global__ void k_qmr2_update(KrylovArgs<Rl> k) {
 template <typename Rl, int G>
 __global__ void __launch_bounds__(G * red_threads<Rl>() + 32, G * red_threads<Rl>() == 512 ? 2 : 4) k_qmr2_post(KrylovArgs<Rl> k) {
     using C = cx<Rl>;
+    dep_wait(k.dep);
     constexpr int RT = red_threads<Rl>();
     namespace cg = cooperative_groups;
     const cg::cluster_group cl = cg::this_cluster();
@@ -725,17 +726,7 @@ template <typename Rl> static bool qmr2_one_kernel(const KrylovArgs<Rl>& k) {
 }
 
 template <typename Rl, int G> static void qmr2_post_launch(const KrylovArgs<Rl>& k, int cl, cudaStream_t st) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(cl, k.S);
-    cfg.blockDim = dim3(G * red_threads<Rl>() + 32);
-    cfg.stream = st;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = cl;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, k_qmr2_post<Rl, G>, k);
+    launch_dep(k.dep, k_qmr2_post<Rl, G>, dim3(cl, k.S), G * red_threads<Rl>() + 32, 0, cl, st, k);
 }
 
 template <typename Rl>

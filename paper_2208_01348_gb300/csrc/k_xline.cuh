@@ -47,6 +47,7 @@ template <typename Rl, int RE, int RO, bool SPLIT>
 __global__ void __launch_bounds__(SPLIT ? 512 : 256, sizeof(Rl) == 4 && RO <= 10 ? (RO <= 6 ? 3 : 2) : 1)
 k_xline(LatticeDev L, MatvecArgs<Rl> a, int lgw) {
     using C = cx<Rl>;
+    dep_wait(a.dep);
     constexpr int LEN = RE * RO, HX = LEN / 2 + 1;
     const int s0 = blockIdx.z * a.spb, s1 = min(a.S, s0 + a.spb);
     const int W = 1 << lgw, ky = blockIdx.y, kz0 = blockIdx.x << lgw;
@@ -159,8 +160,8 @@ template <typename Rl> void launch_xline(const LatticeDev& L, const MatvecArgs<R
     switch (L.Mx) {
 #define XL(RE, RO)                                                                            \
     case RE * RO:                                                                             \
-        if (split) k_xline<Rl, RE, RO, sizeof(Rl) == 8><<<grid, nthr, sm, st>>>(L, b, lgw);  \
-        else k_xline<Rl, RE, RO, false><<<grid, nthr, sm, st>>>(L, b, lgw);                  \
+        if (split) launch_dep(b.dep, k_xline<Rl, RE, RO, sizeof(Rl) == 8>, grid, nthr, sm, 1, st, L, b, lgw); \
+        else launch_dep(b.dep, k_xline<Rl, RE, RO, false>, grid, nthr, sm, 1, st, L, b, lgw);             \
         break;
         EELS_PLANS(XL)
 #undef XL

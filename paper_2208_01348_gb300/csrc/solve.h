@@ -67,6 +67,7 @@ struct KrylovArgs {
     double eps;                    // stop when the (quasi-)residual <= eps ||b||
     const double* eps_sys;         // per-system eps (overrides eps when non-null)
     int max_iter;
+    int dep;                       // the vector kernel starts while the matvec drains (matvec_dep)
 };
 
 // Reduction blocks: how many vector entries each sums, with how many threads.
