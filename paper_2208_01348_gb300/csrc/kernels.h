@@ -50,7 +50,7 @@ void launch_dep(int dep, void (*kernel)(P...), dim3 grid, int threads, size_t sm
     cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
-// Split of a slab pass (k_slab.cu) over the blocks of a cluster: chosen from
+// Split of a slab pass (k_slab.cuh) over the blocks of a cluster: chosen from
 // the lattice alone, so that a system's sums do not depend on the batch.
 struct SlabPlan {
     int CL;                       // blocks per slab

@@ -1,4 +1,4 @@
-// Phases of the fused slab passes (k_slab.cu): one cluster of CL blocks owns
+// Phases of the fused slab passes (k_slab.cuh): one cluster of CL blocks owns
 // the x-slab ix of one (system, component).
 //
 // Forward:  y1, y2   transform the slab's Nz columns along y in place in

@@ -1,4 +1,4 @@
-// Phases of the shared-memory x pass (k_xline.cu): forward x transforms of
+// Phases of the shared-memory x pass (k_xline.cuh): forward x transforms of
 // the three components of W kz-adjacent lines, the symmetric D-hat product
 // and the inverse transforms, for L = RE * RO points.
 //
@@ -6,7 +6,8 @@
 // line sits in row a RE + j.  The middle step reads row j + r RE (r < RO) of
 // the three components, finishes the forward transform (elements
 // kx = j + r RE), multiplies by D-hat and starts the inverse transform on the
-// same elements, all in registers.
+// same elements, all in registers (xline_mid), or a lane does so for one
+// component and takes the products from its neighbours (xline_mid_in, _out).
 #pragma once
 #include "dft.cuh"
 
