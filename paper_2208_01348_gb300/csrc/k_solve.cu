@@ -651,10 +651,10 @@ __global__ void k_qmr2_update(KrylovArgs<Rl> k) {
 //
 // What bounds it: FP64, the pipe (28 instructions an entry); FP32, the L2; for
 // small vectors the launch, the barrier and the scalars' chain.  At most 56
-// registers, so that two clusters share their SMs: 24 systems at one block per
-// SM ran in two rounds (with loads one by one, 1548 us in place of 1285 for 12
-// iterations of 32^3 cells).  Three kernels before: 44 us an iteration of one
-// FP64 system of 2775 entries (now about 10), 28 us of 24 FP32 systems of 51768.
+// registers, so that two clusters share their SMs: at one block per SM, with loads
+// one by one, 24 systems ran in two rounds (FP32 inner solve of 32^3 cells 1548 us,
+// 1285 now).  The three kernels took 44 us an iteration of one FP64 system of 2775
+// entries, this one about 20 (12^3 cells: 54 us an iteration with the matvec's 34).
 template <typename Rl, int G>
 __global__ void __launch_bounds__(G * red_threads<Rl>() + 32, G * red_threads<Rl>() == 512 ? 2 : 4) k_qmr2_post(KrylovArgs<Rl> k) {
     using C = cx<Rl>;
