@@ -715,14 +715,25 @@ __global__ void __launch_bounds__(G * red_threads<Rl>() + 32, G * red_threads<Rl
 
 // One kernel where a cluster of eight SMs does the vectors of a system about as
 // fast as the whole chip would: up to 65536 entries in FP32 (4.6 us of L2
-// traffic per SM) and 32768 in FP64 (0.44 ns of its pipe an entry, against the
-// 12 us or so of three kernels).  By the vector alone: the two forms do not round
-// alike everywhere, and a system's bits do not depend on the batch.  Inner
-// solves, three kernels and one: 24 FP32 systems of 32^3 cells 1469 and 1285 us;
-// whole requests of 16 such systems 77.9 and 65.6 ms, of one FP64 system of 12^3
-// cells 71.6 and 49.8 ms.
+// traffic per SM) and 8192 in FP64 (28 instructions an entry at 19 cycles of an
+// SM's pipe each make 1.1 ns an entry, so 9 us, against the 12 us or so of three
+// kernels).  By the vector alone: the two forms do not round alike everywhere, and
+// a system's bits do not depend on the batch.  us an iteration, three kernels
+// and one, of 1, 4 and 16 systems in FP64:
+//    3000 entries 48.2, 42.6   70.9, 64.2   131, 127
+//    5184         53.9, 51.9   77.8, 76.5   168, 172
+//    6591         65.1, 63.7   103, 101     239, 243
+//    8232         64.6, 65.3   103, 104     241, 247
+//   11253         69.3, 77.6   105, 112     312, 330
+//   31200         121, 147     295, 317     1043, 1077
+// and in FP32 (1, 4 and 24 systems):
+//   24000         35.1, 32.5   46.7, 43.3   124, 120
+//   41472         35.7, 36.8   48.5, 47.8   138, 138
+//   61236         37.9, 37.2   51.7, 51.5   179, 177
+// 24 energies of the 32^3 sphere (51768 entries): inner solve 1469 and 1285 us.
+constexpr int qmr2_one_kernel_max(bool fp64) { return fp64 ? 8192 : 65536; }
 template <typename Rl> static bool qmr2_one_kernel(const KrylovArgs<Rl>& k) {
-    return k.n3 <= (sizeof(Rl) == 4 ? 65536 : 32768);
+    return k.n3 <= qmr2_one_kernel_max(sizeof(Rl) == 8);
 }
 
 template <typename Rl, int G> static void qmr2_post_launch(const KrylovArgs<Rl>& k, int cl, cudaStream_t st) {

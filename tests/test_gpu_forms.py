@@ -1,0 +1,70 @@
+"""GPU: the forms of the QMR update that the length of the vectors chooses."""
+import numpy as np
+import pytest
+
+from paper_2208_01348_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dd():
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2208_01348_gb300 import eelsdda
+    return eelsdda
+
+
+@pytest.fixture()
+def ctx(dd):
+    h = dd.eels_create(0)
+    yield h
+    dd.eels_destroy(h)
+
+
+# 3N entries on both sides of each precision's line between one kernel and three, the
+# padded points of an x pass on both sides of its line between three lanes and one
+@pytest.mark.parametrize("dims,prec,kernels", [((13, 14, 15), "FP64", 4), ((13, 14, 16), "FP64", 6),
+                                               ((2, 3, 3), "FP64", 4), ((16, 16, 16), "FP64", 6),
+                                               ((11, 11, 31), "FP64", 6), ((28, 28, 27), "MIXED", 4),
+                                               ((28, 28, 28), "MIXED", 6)])
+def test_kernels_of_a_qmr2_iteration(dd, ctx, dims, prec, kernels):
+    """The three kernels of the matvec, and one or three for the vectors: 60
+    iterations (ten replays of six) launch what the length of the vectors says, the
+    same iterations of three systems give the bits of each alone, and the solution
+    of a finished solve has the residual it was asked for."""
+    import torch
+    S, eps_h = 3, 1.0 + 0j
+    dd.eels_set_grid(ctx, I.box_occupancy(*dims), 1.5)
+    n = int(np.prod(dims))
+    e = np.array([3.4, 3.7, 4.0])
+    eps_p = np.array([[I.drude(v)] for v in e])
+    p = getattr(dd, "EELS_" + prec)
+    dt, eps = (torch.complex128, 1e-9) if prec == "FP64" else (torch.complex64, 1e-5)
+    g = torch.Generator(device="cuda").manual_seed(2)
+    b = torch.randn((S, 3, n), generator=g, device="cuda", dtype=dt)
+    st = torch.cuda.current_stream().cuda_stream
+
+    def solve(i0, i1, tol, most):
+        dd.eels_prepare_operator(ctx, e[i0:i1], eps_p[i0:i1], np.full(i1 - i0, eps_h))
+        x = torch.zeros_like(b[i0:i1])
+        l0 = dd.eels_kernel_launches()
+        status, iters = dd.eels_krylov_solve_dev(ctx, p, dd.EELS_QMR2, b[i0:i1].data_ptr(), x.data_ptr(), i1 - i0, tol,
+                                                 most, st)
+        torch.cuda.synchronize()
+        return x, status, iters, dd.eels_kernel_launches() - l0
+    x, status, iters, _ = solve(0, S, eps, 3000)
+    assert (status == 1).all()
+    r = torch.zeros_like(x)
+    dd.eels_matvec_dev(ctx, p, x.data_ptr(), r.data_ptr(), S, st)
+    for i in range(S):
+        # the quasi-residual underestimates the residual by at most sqrt(iterations + 1) <= 55
+        assert float(torch.linalg.vector_norm(r[i] - b[i]) / torch.linalg.vector_norm(b[i])) < 55 * eps
+        xi, _, it, n_launch = solve(i, i + 1, eps, 3000)
+        assert it[0] == iters[i] and torch.equal(xi[0], x[i])
+        # three launches start the solve; a replay is six iterations, and the host looks for the end after 1, 2, 4, 8, 8 ...
+        replays, burst = 1, 1
+        while 6 * replays < it[0]:
+            burst = min(8, 2 * burst)
+            replays += burst
+        assert n_launch == 3 + replays * 6 * kernels
