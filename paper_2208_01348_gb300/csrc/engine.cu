@@ -649,6 +649,16 @@ int inner_solve(eels_ctx* c, int S, const eels_opts* o, double eps) {
     // the matvec also returns the per-block partial sums of x^T (A x)
     const bool fused = !bicg;
     k.nblk_a = fused ? matvec_dot_parts(c->L, sizeof(Rl) == 8) : k.nblk;
+    // The body of a conditional node is documented for kernel nodes; programmatic
+    // edges, which dependent launches would leave in it, are not mentioned, so the
+    // device loop's kernels start when the ones before them have ended.
+    const bool dev_loop = o->device_loop != 0;
+    if (dev_loop) k.dep = 0;
+    auto mv = [&](const cx<Rl>* x, cx<Rl>* y) {
+        MatvecArgs<Rl> a = mv_args<Rl>(c, S, x, y, dr_of<Rl>(c), k.active, true);
+        a.no_dep = dev_loop;
+        return a;
+    };
     if (bicg) launch_bicg_init<Rl>(k, st);
     else if (qmr2) launch_qmr2_init<Rl>(k, st);
     else launch_qmr_init<Rl>(k, st);
@@ -666,7 +676,6 @@ int inner_solve(eels_ctx* c, int S, const eels_opts* o, double eps) {
     const void* ek;
     std::memcpy(&ek, &epsv, sizeof(ek));
     key.push_back(ek);
-    const bool dev_loop = o->device_loop != 0;
     key.push_back((const void*)(size_t)dev_loop);
     const int max_chunks = inner_cap(o, sizeof(Rl) == 4) / CHUNK + 2;
     int* chunks = c->counters.as<int>() + 2;
@@ -707,20 +716,20 @@ int inner_solve(eels_ctx* c, int S, const eels_opts* o, double eps) {
         } cguard{st};
         for (int n = 1; n <= CHUNK; ++n) {
             if (bicg) {
-                launch_matvec<Rl>(c->L, mv_args<Rl>(c, S, k.Pb, k.Vb, dr_of<Rl>(c), k.active, true), st);
+                launch_matvec<Rl>(c->L, mv(k.Pb, k.Vb), st);
                 launch_bicg_stage1<Rl>(k, st);
-                launch_matvec<Rl>(c->L, mv_args<Rl>(c, S, k.R, k.Tb, dr_of<Rl>(c), k.active, true), st);
+                launch_matvec<Rl>(c->L, mv(k.R, k.Tb), st);
                 launch_bicg_stage2<Rl>(k, st);
                 continue;
             }
             if (qmr2) {
-                MatvecArgs<Rl> a = mv_args<Rl>(c, S, k.P[0], k.W, dr_of<Rl>(c), k.active, true);
+                MatvecArgs<Rl> a = mv(k.P[0], k.W);
                 a.dot_part = fused ? k.part_a : nullptr;
                 launch_matvec<Rl>(c->L, a, st);
                 launch_qmr2_post_matvec<Rl>(k, fused, st);
                 continue;
             }
-            MatvecArgs<Rl> a = mv_args<Rl>(c, S, k.V[n & 1], k.W, dr_of<Rl>(c), k.active, true);
+            MatvecArgs<Rl> a = mv(k.V[n & 1], k.W);
             a.dot_part = fused ? k.part_a : nullptr;
             launch_matvec<Rl>(c->L, a, st);
             launch_qmr_post_matvec<Rl>(k, n, fused, st);

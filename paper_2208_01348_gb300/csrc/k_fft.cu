@@ -389,7 +389,7 @@ template <typename Rl>
 void launch_matvec(const LatticeDev& L, const MatvecArgs<Rl>& a, cudaStream_t st) {
     // slab (gather, y, z) -> x * D-hat * x -> slab (z, y, scatter)
     MatvecArgs<Rl> b = a;
-    b.dep = matvec_dep(L, a.S, sizeof(Rl) == 8);
+    b.dep = !a.no_dep && matvec_dep(L, a.S, sizeof(Rl) == 8);
     slab_launch_any<Rl>(L, b, false, st);
     xpass_any<Rl>(L, b, st);
     slab_launch_any<Rl>(L, b, true, st);

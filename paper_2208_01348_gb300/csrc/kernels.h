@@ -105,6 +105,7 @@ struct MatvecArgs {
     const float2* Dx;             // FP32 D-hat [slot][Hy][Hz][6][Hx] (register x pass), or nullptr
     int S;
     int dep;                      // generic passes start while the kernel before them drains (set by launch_matvec)
+    int no_dep;                   // the caller's kernels may not (see inner_solve)
     int spb;                      // systems per x-pass block (consecutive systems that usually share a
                                   // D-hat slot: the beams of one energy); 0 or 1: one
 };

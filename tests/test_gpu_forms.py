@@ -1,4 +1,6 @@
-"""GPU: the forms of the QMR update that the length of the vectors chooses."""
+"""GPU: the forms of the QMR update that the length of the vectors chooses, and the
+device loop and stream capture of a request whose kernels start while the ones
+before them drain."""
 import numpy as np
 import pytest
 
@@ -68,3 +70,59 @@ def test_kernels_of_a_qmr2_iteration(dd, ctx, dims, prec, kernels):
             burst = min(8, 2 * burst)
             replays += burst
         assert n_launch == 3 + replays * 6 * kernels
+
+
+@pytest.mark.parametrize("solver", ["QMR2", "QMR", "BICGSTAB"])
+@pytest.mark.parametrize("dims", [(12, 12, 12), (3, 4, 5), (2, 10, 10)])
+def test_device_loop_of_a_request_with_dependent_launches(dd, ctx, dims, solver):
+    """One FP64 point on a lattice whose passes have at most one block per SM: its
+    kernels start while the ones before them drain, in the body of the device loop's
+    WHILE node as in the host's replays, and both loops give the same bits."""
+    dd.eels_set_grid(ctx, I.box_occupancy(*dims), 20.0 / 12)
+    e = np.array([3.4])
+    res = []
+    for loop in (0, 1):
+        o = dd.eels_default_opts(ekin_keV=100.0, precision=dd.EELS_FP64, eps_it=1e-8,
+                                 solver=getattr(dd, "EELS_" + solver), n_dir=162, device_loop=loop)
+        r = dd.eels_solve(ctx, o, e, I.drude(e)[:, None], np.full(1, 1.0 + 0j), np.array([[30.0, 0.0]]), want_p=True)
+        assert r.converged.all()
+        res.append(r)
+    for key in ("p_eels", "p_cl", "p_ext", "p_abs", "p", "residual", "iters"):
+        assert np.array_equal(getattr(res[0], key), getattr(res[1], key)), key
+
+
+@pytest.mark.parametrize("dims,prec", [((12, 12, 12), "FP64"), ((12, 12, 12), "MIXED"), ((11, 11, 31), "FP64")])
+def test_captured_matvec_gives_the_same_bits(dd, ctx, dims, prec):
+    """eels_matvec_dev in a caller's stream capture, after a kernel and after a copy of
+    the caller's, with and without dependent launches: replays on other inputs give
+    the bits of the direct call."""
+    import torch
+    dd.eels_set_grid(ctx, I.box_occupancy(*dims), 1.5)
+    dd.eels_prepare_operator(ctx, [2.4], [[I.drude(2.4)]], [1.0 + 0j])
+    p, dt = getattr(dd, "EELS_" + prec), torch.complex128 if prec == "FP64" else torch.complex64
+    g = torch.Generator(device="cuda").manual_seed(8)
+    n = int(np.prod(dims))
+    src = torch.randn((1, 3, n), generator=g, device="cuda", dtype=dt)
+    x, y, z = torch.zeros_like(src), torch.zeros_like(src), torch.zeros_like(src)
+
+    def step():
+        st = torch.cuda.current_stream().cuda_stream
+        x.copy_(src)
+        dd.eels_matvec_dev(ctx, p, x.data_ptr(), y.data_ptr(), 1, st)
+        x.mul_(2.0)
+        dd.eels_matvec_dev(ctx, p, x.data_ptr(), z.data_ptr(), 1, st)
+    step()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        step()
+    for seed in (1, 2):
+        src.copy_(torch.randn((1, 3, n), generator=g, device="cuda", dtype=dt))
+        step()
+        torch.cuda.synchronize()
+        want_y, want_z = y.clone(), z.clone()
+        y.zero_()
+        z.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(y, want_y) and torch.equal(z, want_z)
