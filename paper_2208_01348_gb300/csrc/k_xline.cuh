@@ -35,14 +35,21 @@ template <typename C> __device__ __forceinline__ C shfl_c(C v, int l) {
     return v;
 }
 
-// SPLIT (FP64, lattices of at most 65536 padded points): the middle step of a
+// SPLIT (FP64, lattices of at most 32768 padded points): the middle step of a
 // line and butterfly is shared by three lanes, one a component.  Such a grid gives
-// a scheduler one or two warps, and a warp's FP64 instruction takes 32 cycles of
-// it (64 where it waits for the one before), so the step's 312 instructions in a
-// row are the kernel: 12^3 cells, one system, 47 -> 39 us a matvec; 16 systems of 11 x 11 x
-// 31 the same either way.  Where there are warps enough it costs more than it
-// gives: 8 systems of 32^3 cells 957 -> 1040 us a matvec, and in FP32 (shuffles on
-// top of the shared-memory accesses) 4 of 79^3 468 -> 660 us.
+// a scheduler one warp or none, and a warp's FP64 instruction takes 64 cycles of
+// its scheduler even when it is alone there (76 with all four of an SM busy), so
+// the step's 312 instructions in a row are the kernel.  Where there are warps enough
+// it costs more than it gives (idle lanes, shuffles).  The lattice alone decides: the
+// compiler fuses the two forms' products differently, and a system's bits must not
+// depend on the batch.  So the line lies where few systems stop gaining, although
+// many systems of the smaller lattices lose.  us a matvec, one lane and three:
+//   12^3 cells   1 system 42.5, 36.7    2: 52.1, 44.6    4: 62.3, 66.4   256: 1713, 1839
+//   14^3         1: 71.9, 54.8          2: 74.6, 61.0    4: 86.2, 90.3
+//   16^3         1: 56.9, 48.7          2: 57.6, 58.2    4: 83.2, 87.6    64: 778, 880
+//   11 x 11 x 31 1: 61.7, 57.6          2: 69.9, 73.9   16: 266, 286
+//   18^3         1: 90.3, 96.5          2: 109, 121     16: 576, 626
+//   20^3         1: 96.5, 103           4: 206, 227    128: 5032, 5668
 template <typename Rl, int RE, int RO, bool SPLIT>
 __global__ void __launch_bounds__(SPLIT ? 512 : 256, sizeof(Rl) == 4 && RO <= 10 ? (RO <= 6 ? 3 : 2) : 1)
 k_xline(LatticeDev L, MatvecArgs<Rl> a, int lgw) {
@@ -136,7 +143,7 @@ template <typename Rl> static size_t xline_smem(const LatticeDev& L, int w) {
 template <typename Rl> bool xline_fits(const LatticeDev& L, int w) { return xline_smem<Rl>(L, w) <= 224 * 1024; }
 
 template <typename Rl> static bool xline_split(const LatticeDev& L) {
-    return sizeof(Rl) == 8 && (long long)L.Mx * L.My * L.Mz <= 65536;
+    return sizeof(Rl) == 8 && (long long)L.Mx * L.My * L.Mz <= 32768;
 }
 
 template <typename Rl> void launch_xline(const LatticeDev& L, const MatvecArgs<Rl>& a, int w, cudaStream_t st) {
