@@ -343,11 +343,16 @@ template <typename Rl> static void slab_launch_any(const LatticeDev& L, const Ma
     launch_slab<Rl>(L, a, inv, st);
 }
 
-// Widest x-pass tile (W lines per component) whose buffer fits a quarter of
-// an SM's shared memory, so that four blocks are resident.
+// Tile width of the x pass before the autotuner has timed it (eels_matvec_dev and
+// eels_krylov_solve_dev without an earlier eels_solve): the widest of 32, 16 and 8
+// lines whose block keeps to 56 KB of shared memory in FP32 and 28 KB in FP64.  Most
+// widths time alike (8 systems of 32^3 cells in FP64 969, 969 and 974 us with 8, 16 and
+// 32 lines), but the wide ones lose where few blocks of them fit: 16 of 24^3 in FP64
+// 982, 981 and 1240, 2 of 64^3 2117, 2180 and 2167, and 4 of 79^3 in FP32 515 us with 8
+// lines and 608 with 16.
 template <typename Rl> static int pick_xpass_w(const LatticeDev& L) {
-    for (int W : {32, 16, 8})
-        if (6 * (size_t)W * L.Mx * sizeof(cx<Rl>) <= 56 * 1024) return W;
+    for (int W : {32, 16})
+        if (xline_smem<Rl>(L, W) <= (sizeof(Rl) == 4 ? 56 : 28) * 1024) return W;
     return 8;
 }
 

@@ -137,7 +137,7 @@ k_xline(LatticeDev L, MatvecArgs<Rl> a, int lgw) {
     }
 }
 
-template <typename Rl> static size_t xline_smem(const LatticeDev& L, int w) {
+template <typename Rl> size_t xline_smem(const LatticeDev& L, int w) {
     return (size_t)(L.Mx + 3 * w * L.Mx + (sizeof(Rl) == 4 ? 6 * w * (L.Mx / 2 + 1) : 0)) * sizeof(cx<Rl>);
 }
 template <typename Rl> bool xline_fits(const LatticeDev& L, int w) { return xline_smem<Rl>(L, w) <= 224 * 1024; }

@@ -163,6 +163,7 @@ unsigned int wait_timeouts();
 
 // Shared-memory x pass of any length, w kz-adjacent lines per block (a power
 // of two; narrower when the grid would leave SMs idle).
+template <typename Rl> size_t xline_smem(const LatticeDev& L, int w);   // shared memory of such a block
 template <typename Rl> bool xline_fits(const LatticeDev& L, int w);
 template <typename Rl> void launch_xline(const LatticeDev& L, const MatvecArgs<Rl>& a, int w, cudaStream_t st);
 template <typename Rl> void prepare_xline_kernels();
