@@ -69,6 +69,37 @@ __device__ __forceinline__ void slab_tables(const LatticeDev& L, const MatvecArg
     }
 }
 
+// The rows of a thread's z transforms: those of its warp (G at a time), or, with
+// the wide form, of its block (G per warp), whose threads then take the butterflies
+// of all of them, one row after another.  The FP64 pipe takes a warp's instruction in
+// the same time however many of its lanes work, and a warp's own rows leave lanes idle
+// wherever G Ro or G Re are not near multiples of 32: with 250 points (radices 10 and
+// 25) and G = 1 the slab passes of three systems of 12 x 96 x 125 cells issued 14.4 M and
+// 15.2 M FP64 instructions and took 1.07 and 1.05 ms; shared by blocks of twelve warps
+// with G = 2 they issue 6.8 M and 7.6 M and take 0.48 and 0.54 ms.  The bits are the
+// same.  Two block barriers a turn are what it costs, so slabs whose rows fill their
+// warps keep the private form (make_slab_plan).
+template <typename Rl> struct SlabRows {
+    int lane, nl;                 // place among the threads that share rows
+    int first, step, g;           // rows of a turn, and of the next one
+    size_t tile;                  // exchange tile
+    bool wide;
+    __device__ SlabRows(const SlabPlan& p, const Plan2& qz) {
+        const int warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+        wide = sizeof(Rl) == 8 && p.wide;
+        lane = wide ? threadIdx.x : threadIdx.x & 31;
+        nl = wide ? blockDim.x : 32;
+        step = nwarp * p.G;
+        first = wide ? 0 : warp * p.G;
+        g = wide ? step : p.G;
+        tile = (size_t)first * qz.Ro * (qz.Re + 1);
+    }
+    __device__ void sync() const {
+        if (wide) __syncthreads();
+        else __syncwarp();
+    }
+};
+
 template <typename Rl, bool CLUSTER>
 __global__ void __launch_bounds__(sizeof(Rl) == 4 ? 768 : 512, 1) k_slab_fwd(LatticeDev L, MatvecArgs<Rl> a) {
     using C = cx<Rl>;
@@ -122,25 +153,24 @@ __global__ void __launch_bounds__(sizeof(Rl) == 4 ? 768 : 512, 1) k_slab_fwd(Lat
     }
     if (CLUSTER) cg::this_cluster().sync();
     else __syncthreads();
-    // z transforms of this block's rows, G per warp
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
-    const int lp = L.qz.Ro * (L.qz.Re + 1);
-    C* T = m.T + (size_t)warp * sp.G * lp;
+    // z transforms of this block's rows
+    const SlabRows<Rl> rows(sp, L.qz);
+    C* T = m.T + rows.tile;
     C* U = a.U + (((size_t)s * 3 + c) * L.My * L.Nx + ix) * (size_t)L.Mz;
     const size_t urow = (size_t)L.Nx * L.Mz;
-    for (int row = sc.r0 + warp * sp.G; row < sc.r0 + sc.nrow; row += nwarp * sp.G) {
-        const int g = min(sp.G, sc.r0 + sc.nrow - row);
+    for (int row = sc.r0 + rows.first; row < sc.r0 + sc.nrow; row += rows.step) {
+        const int g = min(rows.g, sc.r0 + sc.nrow - row);
         auto out = [&](int q, int kz) -> C* { return U + (size_t)(row + q) * urow + kz; };
         if (CLUSTER) {
             auto in = [&](int q, int j, int dz) -> const C* {
                 const int z = j + dz, o = (int)sp.dcpc.div(z);
                 return cg::this_cluster().map_shared_rank(m.S, o) + (row + q) * sp.sls + z - o * sp.cpc;
             };
-#define Z1(R) case R: slab_z1<R, C>(rz, Nz, g, T, lane, in); break;
+#define Z1(R) case R: slab_z1<R, C>(rz, Nz, g, T, rows.lane, in, rows.nl); break;
             EELS_SWITCH_RE(L.qz.Re, Z1)
 #undef Z1
-            __syncwarp();
-#define Z2(R) case R: slab_z2<R, C>(rz, g, T, m.twz, lane, out); break;
+            rows.sync();
+#define Z2(R) case R: slab_z2<R, C>(rz, g, T, m.twz, rows.lane, out, rows.nl); break;
             EELS_SWITCH_RO(L.qz.Ro, Z2)
 #undef Z2
         } else {
@@ -148,14 +178,14 @@ __global__ void __launch_bounds__(sizeof(Rl) == 4 ? 768 : 512, 1) k_slab_fwd(Lat
             auto in = [&](int q, int j, int dz) -> const C* { return Sr + q * sp.sls + j + dz; };
 #define Z(RE, RO)                                                                     \
     case RE * RO:                                                                     \
-        slab_z1<RE, C>(CtPlan<RE, RO>{}, Nz, g, T, lane, in);                         \
-        __syncwarp();                                                                 \
-        slab_z2<RO, C>(CtPlan<RE, RO>{}, g, T, m.twz, lane, out);                     \
+        slab_z1<RE, C>(CtPlan<RE, RO>{}, Nz, g, T, rows.lane, in, rows.nl);       \
+        rows.sync();                                                                  \
+        slab_z2<RO, C>(CtPlan<RE, RO>{}, g, T, m.twz, rows.lane, out, rows.nl);   \
         break;
             switch (L.Mz) { EELS_PLANS(Z) default: break; }
 #undef Z
         }
-        __syncwarp();
+        rows.sync();
     }
     if (CLUSTER) cg::this_cluster().sync();           // other blocks may still read this block's S
 }
@@ -183,12 +213,12 @@ __global__ void __launch_bounds__(sizeof(Rl) == 4 ? 768 : 512, 1) k_slab_inv(Lat
     const FastDiv dcol = fast_div(sc.ncol);
     // inverse z transforms of this block's rows of U, first Nz outputs into the columns' owners
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
-    const int lp = L.qz.Ro * (L.qz.Re + 1);
-    C* T = m.T + (size_t)warp * sp.G * lp;
+    const SlabRows<Rl> rows(sp, L.qz);
+    C* T = m.T + rows.tile;
     const C* U = a.U + (((size_t)s * 3 + c) * L.My * L.Nx + ix) * (size_t)L.Mz;
     const size_t urow = (size_t)L.Nx * L.Mz;
-    for (int row = sc.r0 + warp * sp.G; row < sc.r0 + sc.nrow; row += nwarp * sp.G) {
-        const int g = min(sp.G, sc.r0 + sc.nrow - row);
+    for (int row = sc.r0 + rows.first; row < sc.r0 + sc.nrow; row += rows.step) {
+        const int g = min(rows.g, sc.r0 + sc.nrow - row);
         auto in = [&](int q, int kz) -> const C* { return U + (size_t)(row + q) * urow + kz; };
         if (CLUSTER) {
             const RtPlan rz{L.qz};
@@ -196,11 +226,11 @@ __global__ void __launch_bounds__(sizeof(Rl) == 4 ? 768 : 512, 1) k_slab_inv(Lat
                 const int z = j + dz, o = (int)sp.dcpc.div(z);
                 return cg::this_cluster().map_shared_rank(m.S, o) + (row + q) * sp.sls + z - o * sp.cpc;
             };
-#define Z1(R) case R: slab_z1i<R, C>(rz, g, T, m.twz, lane, in); break;
+#define Z1(R) case R: slab_z1i<R, C>(rz, g, T, m.twz, rows.lane, in, rows.nl); break;
             EELS_SWITCH_RO(L.qz.Ro, Z1)
 #undef Z1
-            __syncwarp();
-#define Z2(R) case R: slab_z2i<R, C>(rz, Nz, g, T, lane, out); break;
+            rows.sync();
+#define Z2(R) case R: slab_z2i<R, C>(rz, Nz, g, T, rows.lane, out, rows.nl); break;
             EELS_SWITCH_RE(L.qz.Re, Z2)
 #undef Z2
         } else {
@@ -208,14 +238,14 @@ __global__ void __launch_bounds__(sizeof(Rl) == 4 ? 768 : 512, 1) k_slab_inv(Lat
             auto out = [&](int q, int j, int dz) -> C* { return Sr + q * sp.sls + j + dz; };
 #define Z(RE, RO)                                                                     \
     case RE * RO:                                                                     \
-        slab_z1i<RO, C>(CtPlan<RE, RO>{}, g, T, m.twz, lane, in);                     \
-        __syncwarp();                                                                 \
-        slab_z2i<RE, C>(CtPlan<RE, RO>{}, Nz, g, T, lane, out);                       \
+        slab_z1i<RO, C>(CtPlan<RE, RO>{}, g, T, m.twz, rows.lane, in, rows.nl);                     \
+        rows.sync();                                                                  \
+        slab_z2i<RE, C>(CtPlan<RE, RO>{}, Nz, g, T, rows.lane, out, rows.nl);     \
         break;
             switch (L.Mz) { EELS_PLANS(Z) default: break; }
 #undef Z
         }
-        __syncwarp();
+        rows.sync();
     }
     if (CLUSTER) cg::this_cluster().sync();
     else __syncthreads();

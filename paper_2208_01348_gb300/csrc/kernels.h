@@ -58,6 +58,7 @@ struct SlabPlan {
     int sls;                      // row stride of a block's columns S[My][sls]
     int G;                        // rows a warp transforms at a time
     int nthr;
+    int wide;                     // FP64: the block's warps share the rows of all of them
     FastDiv dcpc;                 // division by cpc
 };
 

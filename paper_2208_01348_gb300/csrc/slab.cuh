@@ -12,7 +12,9 @@
 //                    scattered.
 // A warp takes G rows at a time through a private exchange tile
 // T[G][Ro][Re + 1] (the odd stride keeps both steps' accesses off each
-// other's banks), so the z phase needs no block barrier.
+// other's banks), so the z phase needs no block barrier; with the wide form
+// (large FP64 slabs, SlabRows in k_slab.cuh) the block's warps share G rows each
+// and their tiles, and two block barriers follow a turn.
 //
 // What bounds it: instruction issue and the latency of the gather and of U in
 // FP32 (the rod's 48 x 144 slabs, 256 systems: 0.47 ms forward and 0.54 ms
@@ -119,12 +121,12 @@ HD void slab_y2i(const SlabCtx<Rl>& s, P p, FastDiv dcol, int n, int tid, int nt
 }
 
 // ---------------------------------------------------------------- z phase
-// g rows of a warp from row0 on; the lanes share their butterflies.  in and
+// g rows; nl lanes (a warp, or a whole block) share their butterflies.  in and
 // out return the address of element z (or kz) of row q.
 template <int R, typename C, class P, class In>
-HD void slab_z1(P p, int n, int g, C* T, int lane, In in) {
+HD void slab_z1(P p, int n, int g, C* T, int lane, In in, int nl = 32) {
     const int total = g * p.Ro(), lp = p.Ro() * (R + 1);
-    for (int t = lane; t < total; t += 32) {
+    for (int t = lane; t < total; t += nl) {
         const int q = p.div_ro(t), j = t - q * p.Ro();
         C v[R];
 #pragma unroll
@@ -139,9 +141,9 @@ HD void slab_z1(P p, int n, int g, C* T, int lane, In in) {
     }
 }
 template <int R, typename C, class P, class Out>
-HD void slab_z2(P p, int g, const C* T, const C* tw, int lane, Out out) {
+HD void slab_z2(P p, int g, const C* T, const C* tw, int lane, Out out, int nl = 32) {
     const int total = g * p.Re(), lp = R * (p.Re() + 1);
-    for (int t = lane; t < total; t += 32) {
+    for (int t = lane; t < total; t += nl) {
         const int q = p.div_re(t), j = t - q * p.Re();
         const C* d = T + q * lp + j;
         const C* w = tw + j;
@@ -158,9 +160,9 @@ HD void slab_z2(P p, int g, const C* T, const C* tw, int lane, Out out) {
     }
 }
 template <int R, typename C, class P, class In>
-HD void slab_z1i(P p, int g, C* T, const C* tw, int lane, In in) {
+HD void slab_z1i(P p, int g, C* T, const C* tw, int lane, In in, int nl = 32) {
     const int total = g * p.Re(), lp = R * (p.Re() + 1);
-    for (int t = lane; t < total; t += 32) {
+    for (int t = lane; t < total; t += nl) {
         const int q = p.div_re(t), j = t - q * p.Re();
         const C* i = in(q, j);
         const C* w = tw + j;
@@ -174,9 +176,9 @@ HD void slab_z1i(P p, int g, C* T, const C* tw, int lane, In in) {
     }
 }
 template <int R, typename C, class P, class Out>
-HD void slab_z2i(P p, int n, int g, const C* T, int lane, Out out) {
+HD void slab_z2i(P p, int n, int g, const C* T, int lane, Out out, int nl = 32) {
     const int total = g * p.Ro(), lp = p.Ro() * (R + 1);
-    for (int t = lane; t < total; t += 32) {
+    for (int t = lane; t < total; t += nl) {
         const int q = p.div_ro(t), j = t - q * p.Ro();
         const C* d = T + q * lp + j * (R + 1);
         C v[R];

@@ -1,9 +1,13 @@
-"""GPU: the forms of the QMR update that the length of the vectors chooses, and the
-device loop and stream capture of a request whose kernels start while the ones
-before them drain."""
+"""GPU: the forms of the matvec and of the QMR update that the size of a request
+chooses, and the device loop and stream capture of a request whose kernels start
+while the ones before them drain.
+
+Tolerances against the oracle are those of the matvec elsewhere (FP64 1e-12 in the
+relative 2-norm)."""
 import numpy as np
 import pytest
 
+from oracle import green, run
 from paper_2208_01348_gb300 import inputs as I
 
 pytestmark = pytest.mark.gpu
@@ -24,6 +28,26 @@ def ctx(dd):
     dd.eels_destroy(h)
 
 
+# FP64 slabs whose rows a block shares: clusters of two, four and eight blocks,
+# lattices shorter than their padding, rows that do not fill the last turn
+@pytest.mark.parametrize("dims", [(36, 48, 48), (40, 24, 96), (26, 36, 69), (12, 48, 108), (3, 48, 71), (2, 48, 107),
+                                  (1, 80, 125), (1, 125, 40), (1, 120, 119), (2, 128, 100)])
+def test_fp64_rows_shared_by_a_block_equal_fft_oracle(dd, ctx, dims):
+    eps_h, d_nm, e_eV = 2.1 + 0.1j, 1.5, 2.3
+    occ = I.box_occupancy(*dims)
+    rng = np.random.default_rng(dims[1] * 1000 + dims[2])
+    occ *= (rng.random(occ.shape) < 0.8).astype(np.uint8)
+    occ.flat[0] = 1
+    dd.eels_set_grid(ctx, occ, d_nm)
+    eps_p = [I.drude(e_eV)]
+    pt = run.setup(*dims, d_nm, occ, e_eV, eps_p, eps_h, (300.0, 300.0), ekin_keV=100.0)
+    op = green.FFTOperator(pt.idx, pt.n_axes, pt.d, pt.k, pt.alpha)
+    x = I.random_complex((1, len(pt.r), 3), seed=3)
+    y = dd.eels_apply_matrix(ctx, dd.EELS_FP64, e_eV, eps_p, eps_h, x)
+    ref = op.matvec(x[0])
+    assert np.linalg.norm(y[0] - ref) < 1e-12 * np.linalg.norm(ref)
+
+
 # 3N entries on both sides of each precision's line between one kernel and three, the
 # padded points of an x pass on both sides of its line between three lanes and one
 @pytest.mark.parametrize("dims,prec,kernels", [((13, 14, 15), "FP64", 4), ((13, 14, 16), "FP64", 6),
@@ -31,10 +55,9 @@ def ctx(dd):
                                                ((11, 11, 31), "FP64", 6), ((28, 28, 27), "MIXED", 4),
                                                ((28, 28, 28), "MIXED", 6)])
 def test_kernels_of_a_qmr2_iteration(dd, ctx, dims, prec, kernels):
-    """The three kernels of the matvec, and one or three for the vectors: 60
-    iterations (ten replays of six) launch what the length of the vectors says, the
-    same iterations of three systems give the bits of each alone, and the solution
-    of a finished solve has the residual it was asked for."""
+    """The three kernels of the matvec, and one or three for the vectors: a solve
+    launches what the length of the vectors says, reaches the residual it was asked
+    for, and three systems together have the bits of each alone."""
     import torch
     S, eps_h = 3, 1.0 + 0j
     dd.eels_set_grid(ctx, I.box_occupancy(*dims), 1.5)
