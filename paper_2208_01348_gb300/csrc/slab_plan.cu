@@ -31,21 +31,22 @@ Plan2 make_plan2(int L) {
 // waits at its barriers with nothing beside it (the rod's 48 x 144 slabs: 0.80
 // ms with one block of 24 warps, 0.47 ms with three of 8).
 //
-// FP32, and FP64 slabs of up to 8192 points: more than one block per slab pays
-// cluster barriers and remote shared-memory accesses (+70 % in FP32, +30 % in FP64):
-// only where one does not fit, or too few of its warps do.  In a sweep over lattices
-// of 11 to 96 cells the splits chosen here came within 6 % of the fastest of 100 per
-// lattice.
+// FP32, and FP64 slabs of up to 8192 points (4096 with 128 and more along z): more
+// than one block per slab pays cluster barriers and remote shared-memory accesses
+// (+70 % in FP32, +30 % in FP64): only where one does not fit, or too few of its
+// warps do.  In a sweep over lattices of 11 to 96 cells the splits chosen here came
+// within 6 % of the fastest of 100 per lattice.
 //
 // Larger FP64 slabs are bound by the FP64 pipe, where idle lanes cost as much as busy
 // ones: the z transforms may run over the rows of a whole block (wide), warps without
 // a column issue nothing, and two or four blocks per slab cost next to nothing (eight
 // 30 %).  Slabs that leave some of the 152 SMs idle take more blocks: one and a half
 // systems are reckoned with, since the lattice alone decides.  (By this rule smaller
-// slabs gain with one or two systems and lose up to 14 % with more.)  Fitted to 91
-// sets of lattice and batch, up to 400 splits each: 0.9 % above the fastest matvec on
-// average, 10 % at worst.  us a matvec with the rule of the small slabs, as chosen
-// here, and with the five passes of run-time stages that such lattices had before:
+// slabs of short z lines gain with one or two systems and lose up to 14 % with more.)
+// Fitted to 91 sets of lattice and batch, up to 400 splits each: 0.9 % above the
+// fastest matvec on average, 10 % at worst.  us a matvec with the rule of the small
+// slabs, as chosen here, and with the five passes of run-time stages that such
+// lattices had before:
 //   12 x  96 x 125 cells, 3 systems  2991, 1889, 1867
 //   12 x 120 x 120                   2832, 2074, 2204
 //   12 x  48 x 108                    855,  760,  784
@@ -55,7 +56,7 @@ Plan2 make_plan2(int L) {
 // along z (radices 10 and 25) are what stays behind those.
 SlabPlan make_slab_plan(const LatticeDev& L, size_t el) {
     const Plan2 &y = L.qy, &z = L.qz;
-    const bool fp64 = el == sizeof(double2), large = fp64 && L.My * L.Mz > 8192;
+    const bool fp64 = el == sizeof(double2), large = fp64 && (L.My * L.Mz > 8192 || (L.My * L.Mz >= 4096 && L.Mz >= 128));
     const int most = fp64 ? 512 : 768, enough = large ? 12 : most / 32;
     const double slowest = large ? 6 : 4;
     auto remote = [&](int cl) { return cl == 1 ? 1.0 : !fp64 ? 1.7 : !large || cl == 8 ? 1.3 : cl == 2 ? 1.03 : 1.0; };
