@@ -353,8 +353,10 @@ struct Plan2 {
 };
 
 // The plan (Re, Ro) of every padded length (the even 7-smooth numbers up to
-// 256): the pair with the smallest max(2 Re, 3 Ro), because a thread of the x
-// pass holds three lines in its middle step.
+// 256): the pair of the radices below with the smallest max(2 Re, 3 Ro), because
+// a thread of the x pass holds three lines in its middle step.  Ro = 2 is not
+// among them: it would serve L = 4 and 8 alone, (2, 2) and (4, 2), whose passes
+// take no longer than their launches.
 #define EELS_PLANS(X) \
     X(2, 1) X(4, 1) X(2, 3) X(2, 4) X(2, 5) X(4, 3) X(2, 7) X(4, 4) X(6, 3) X(4, 5) X(6, 4) X(4, 7) X(6, 5) \
     X(8, 4) X(6, 6) X(8, 5) X(6, 7) X(8, 6) X(10, 5) X(6, 9) X(8, 7) X(10, 6) X(8, 8) X(10, 7) X(12, 6) \

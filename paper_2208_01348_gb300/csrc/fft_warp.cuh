@@ -17,10 +17,12 @@
 
 namespace eels {
 
-// Transpose tile strides (8-byte units), even and line -> 4 (mod 16): a lane
-// writes its row in 16-byte pieces (half the instructions of 8-byte stores at
-// the same wavefronts), and the 8 lanes of each quarter-warp store as well as
-// the 16 of each half-warp load fall on distinct banks.
+// Transpose tile strides (8-byte units).  64 points: even, line -> 4 (mod 16):
+// a lane writes its row in 16-byte pieces (half the instructions of 8-byte stores
+// at the same wavefronts), and the 8 lanes of each quarter-warp store as well as
+// the 16 of each half-warp load fall on distinct banks.  128 points: line -> 4,
+// lane -> 1 (mod 16), 8-byte stores: the 16 lanes of each half-warp store and of
+// each half-warp load fall on distinct banks.
 constexpr int R64_QS = 84, R64_PS = 10, R64_TILE = 4 * R64_QS;
 constexpr int R128_QS = 148, R128_PS = 17, R128_TILE = 4 * R128_QS;
 
@@ -145,16 +147,6 @@ __device__ __forceinline__ void fft128_warp_t(float2 (&v)[16], float2* tile, int
         v[2 * k2] = a[k2];
         v[2 * k2 + 1] = b[k2];
     }
-}
-
-// Twiddles from a shared table tw[t] = exp(-2 pi i t / L).
-template <bool INV, bool HIN = false>
-__device__ __forceinline__ void fft64_warp(float2 (&v)[8], float2* tile, int q, int p, const float2* tw) {
-    fft64_warp_t<INV, HIN>(v, tile, q, p, [&](int k) { return tw[p * k]; });
-}
-template <bool INV, bool HIN = false>
-__device__ __forceinline__ void fft128_warp(float2 (&v)[16], float2* tile, int q, int p, const float2* tw) {
-    fft128_warp_t<INV, HIN>(v, tile, q, p, [&](int k) { return tw[p * k]; });
 }
 
 // One transform of L = 8 R points per line: the 64- or 128-point routine.

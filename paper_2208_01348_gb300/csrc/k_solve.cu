@@ -58,8 +58,8 @@ __device__ __forceinline__ void block_sum(T (&v)[K]) {
 
 // Sums four values over the warp: every lane receives the total of v[lane & 3].
 // Lanes trade the values they drop, so the tree takes 6 additions where four
-// separate trees take 20: an FP64 addition of a warp occupies the pipe for 16
-// cycles.
+// separate trees take 20: an FP64 addition of a warp occupies an SM's pipe for 19
+// cycles (red_chunk in solve.h).
 template <typename T> __device__ __forceinline__ T warp_sum4(const T (&v)[4]) {
     const int lane = threadIdx.x & 31;
     const bool hi = lane & 1, up = lane & 2;
@@ -489,8 +489,8 @@ struct Qmr2Coef {
 
 // The scalars of iteration n, in three parts by one warp (every lane the same
 // inputs).  A warp's FP64 instruction takes its scheduler's share of the pipe
-// for 64 cycles whether one lane works or 32, so a division or a root costs
-// half a microsecond and the chain between the sums of v~ and the update is what
+// for 64 cycles or more whether one lane works or 32, so a division or a root
+// costs half a microsecond and the chain between the sums of v~ and the update is what
 // the kernel waits for: Qmr2Pre holds what eps_n = p_n^T A p_n alone decides,
 // qmr2_coefs takes one reciprocal root for both of its arguments and shares the
 // products among the lanes, and qmr2_finish, what only the next iteration and

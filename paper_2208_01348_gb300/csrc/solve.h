@@ -72,10 +72,12 @@ struct KrylovArgs {
 
 // Reduction blocks: how many vector entries each sums, with how many threads.
 // They depend on the vector alone, so a system's sums do not depend on the
-// batch.  FP64 vectors take small blocks: an SM issues one FP64 warp
-// instruction every 16 cycles, so 4096 entries on one SM take 20 us where the
-// whole chip needs a few hundred ns; long ones take fewer (every block of the
-// next kernel adds all partial sums).
+// batch.  FP64 vectors take small blocks: 4096 entries on one SM take 20 us where
+// the whole chip needs a few hundred ns; long ones take fewer (every block of the
+// next kernel adds all partial sums).  The FP64 pipe, measured with chains of fused
+// multiply-adds on one SM: a scheduler by itself gets a warp instruction through
+// every 64 cycles, dependent or not, and all four together one every 19 (76 each),
+// against 16 by the rate that profilers count the pipe's activity against.
 __host__ __device__ constexpr int red_chunk(int n3, bool fp64) {
     return !fp64 || n3 > 131072 ? 4096 : n3 > 32768 ? 1024 : 256;
 }
