@@ -62,8 +62,8 @@ CPU_SAMPLE = {"spectrum": (100, 0, None), "small": (0, 0, None),
 # measured on the workload TRAFFIC_WORKLOAD with kernel sources that hash to
 # TRAFFIC_SRC_HASH; reported as null for other workloads (other FFT sizes,
 # other kernels) and when the kernel sources differ from the measured ones.
-TRAFFIC_BYTES_PER_SYSTEM = 115_766_848   # 1,852,269,568 B over 16 systems, 128^3 FFT
-TRAFFIC_SRC_HASH = "1ee292d212c5f1ea"
+TRAFFIC_BYTES_PER_SYSTEM = 115_716_448   # 1,851,463,168 B over 16 systems, 128^3 FFT
+TRAFFIC_SRC_HASH = "b8ab6b2277a19112"
 TRAFFIC_WORKLOAD = "cherenkov"
 
 

@@ -652,9 +652,9 @@ __global__ void k_qmr2_update(KrylovArgs<Rl> k) {
 // What bounds it: FP64, the pipe (28 instructions an entry); FP32, the L2; for
 // small vectors the launch, the barrier and the scalars' chain.  At most 56
 // registers, so that two clusters share their SMs: at one block per SM, with loads
-// one by one, 24 systems ran in two rounds (FP32 inner solve of 32^3 cells 1548 us,
-// 1285 now).  The three kernels took 44 us an iteration of one FP64 system of 2775
-// entries, this one about 20 (12^3 cells: 54 us an iteration with the matvec's 34).
+// one by one, 24 FP32 systems of 32^3 cells ran in two rounds (an inner solve took
+// 1.2 times as long).  An iteration of one FP64 system of 3000 entries takes 42.6 us
+// with it and 48.2 with the three kernels, the matvec's three included.
 template <typename Rl, int G>
 __global__ void __launch_bounds__(G * red_threads<Rl>() + 32, G * red_threads<Rl>() == 512 ? 2 : 4) k_qmr2_post(KrylovArgs<Rl> k) {
     using C = cx<Rl>;
@@ -730,7 +730,8 @@ __global__ void __launch_bounds__(G * red_threads<Rl>() + 32, G * red_threads<Rl
 //   24000         35.1, 32.5   46.7, 43.3   124, 120
 //   41472         35.7, 36.8   48.5, 47.8   138, 138
 //   61236         37.9, 37.2   51.7, 51.5   179, 177
-// 24 energies of the 32^3 sphere (51768 entries): inner solve 1469 and 1285 us.
+// Inner solves of 4, 24 and 200 energies of the 32^3 sphere (51768 entries, FP32): 582,
+// 1231 and 7070 us with three kernels, 552, 1215 and 7200 with one.
 constexpr int qmr2_one_kernel_max(bool fp64) { return fp64 ? 8192 : 65536; }
 template <typename Rl> static bool qmr2_one_kernel(const KrylovArgs<Rl>& k) {
     return k.n3 <= qmr2_one_kernel_max(sizeof(Rl) == 8);
